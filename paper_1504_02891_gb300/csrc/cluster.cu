@@ -278,7 +278,7 @@ __global__ void __launch_bounds__(NTHREADS) k_cluster_alg1(ClusterArgs A) {
         LineSym<float, RFFT::F> sym;
         sym.c2 = 0.5f / n0;
         sym.dl = A.dlam0;
-        ExRow<C, RFFT::P> ex{f0 + lq * RFFT::P, fbuf, 1 + lq, RTPL};
+        ExRow<C, RFFT::P> ex{f0 + lq * RFFT::P, fbuf, 1 + lq, RTPL, nullptr};
         for (int lb = 0; lb < nlines; lb += RLPC) {
           // every lane of a warp runs the transform (its exchanges are warp
           // barriers); lines past the CTA's rows carry zeros and store nothing
@@ -328,7 +328,7 @@ __global__ void __launch_bounds__(NTHREADS) k_cluster_alg1(ClusterArgs A) {
         LineSym<float, RFFT::F> sym;
         sym.c2 = 0.5f / n1;
         sym.dl = A.dlam1;
-        ExRow<C, RFFT::P> ex{f0 + lq * RFFT::P, fbuf, 1 + lq, RTPL};
+        ExRow<C, RFFT::P> ex{f0 + lq * RFFT::P, fbuf, 1 + lq, RTPL, nullptr};
         for (int lb = 0; lb < nlines; lb += RLPC) {
           const int line = lb + lq;
           const bool act = line < nlines;

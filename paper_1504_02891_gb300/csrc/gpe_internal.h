@@ -64,7 +64,7 @@ template <typename T>
 struct GridDev {
   using C = typename C2t<T>::type;
   T* V = nullptr;
-  C* tw[3] = {nullptr, nullptr, nullptr};
+  C* tw[3] = {nullptr, nullptr, nullptr};   // float64: the fixed-point table (PassGeom::twf) follows in the same allocation
   T* lam[3] = {nullptr, nullptr, nullptr};
   T* coord[3] = {nullptr, nullptr, nullptr};
   PassGeom<T> geom[3];

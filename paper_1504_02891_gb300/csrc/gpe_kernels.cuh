@@ -171,6 +171,7 @@ struct PassGeom {
   int tiles;            // tiles per instance
   int xt;               // axes 1,2: tiles along x
   const typename C2t<T>::type* tw;  // e^{-2 pi i k / F}
+  const int4* twf;      // float64 grids: the same as 62-bit fractions, (re hi, re lo, im hi, im lo)
   const T* lam;         // wavenumber of FFT index m
   T c2, c1;             // symbol = c2*lam^2 + c1*coord*lam  (1/F folded in)
   T dlam;               // lam of FFT index m = dlam * p(m), p(m) = m or m - F

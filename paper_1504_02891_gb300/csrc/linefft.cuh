@@ -15,9 +15,22 @@
 
 namespace gpe {
 
+// The line symbol: c2 lam^2 + c1c lam, lam = dl * (m or m - F).
+template <typename T, int F>
+struct LineSym {
+  T c2, c1c, dl;
+  __device__ __forceinline__ T operator()(int m) const {
+    const T lm = dl * (T)(m < (F >> 1) ? m : m - F);
+    return (c2 * lm + c1c) * lm;
+  }
+};
+
+// Float32 (the float64 line operator is in fixfft.cuh).
 template <typename T, int LF>
 struct LineFFT {
   using C = typename C2t<T>::type;
+  using X = C;                                      // what the exchanges move
+  using Tw = C;                                     // twiddle table entry
   static constexpr int F = 1 << LF;
   static constexpr int TPL = F / 8;                 // threads per line
   static constexpr int N8 = LF / 3;                 // radix-8 stages
@@ -25,49 +38,35 @@ struct LineFFT {
   // line pitch of the exchange buffers (complex): room for F points, and
   // = 8 (mod 16) so that neighbouring lines start half a bank row apart
   static constexpr int P = ((F + F / 16 + 15) & ~15) + 8;
-  // twiddles e^{-2 pi i n / F} come from the table tws (shared memory); in
-  // float32 the thread's 13-17 twiddles are also kept in registers
-  static constexpr bool TW_REG = sizeof(T) == 4;
-  C w8[TW_REG && N8 > 1 ? N8 - 1 : 1][7];
-  C wt[TW_REG ? 6 : 1];
-  const C* tws;
+  // the thread's 13-17 twiddles e^{-2 pi i n / F} are kept in registers
+  C w8[N8 > 1 ? N8 - 1 : 1][7];
+  C wt[6];
   int j;
 
   // twiddle r of radix-8 stage st (>= 1): e^{-2 pi i r k / (8 Ns)}, k = j mod Ns
-  __device__ __forceinline__ C tw8(int st, int r) const {
-    if constexpr (TW_REG) return w8[st - 1][r - 1];
-    const int Ns = 1 << (3 * st);
-    return tws[(r * (j & (Ns - 1))) << (LF - 3 - 3 * st)];
-  }
+  __device__ __forceinline__ C tw8(int st, int r) const { return w8[st - 1][r - 1]; }
   // tail twiddles: radix-4 (i = r - 1 for butterfly j, r + 2 for j + F/8),
   // radix-2 (i = u)
-  __device__ __forceinline__ C twt(int i) const {
-    if constexpr (TW_REG) return wt[i];
-    if constexpr (TAIL == 2) return tws[i < 3 ? (i + 1) * j : (i - 2) * (j + TPL)];
-    return tws[j + i * TPL];
-  }
+  __device__ __forceinline__ C twt(int i) const { return wt[i]; }
 
-  __device__ __forceinline__ void init(int jj, const C* table) {
+  __device__ __forceinline__ void init(int jj, const Tw* table) {
     j = jj;
-    tws = table;
-    if constexpr (TW_REG) {
 #pragma unroll
-      for (int st = 1; st < N8; ++st) {
-        const int Ns = 1 << (3 * st);
-        const int k = j & (Ns - 1);
+    for (int st = 1; st < N8; ++st) {
+      const int Ns = 1 << (3 * st);
+      const int k = j & (Ns - 1);
 #pragma unroll
-        for (int r = 1; r < 8; ++r) w8[st - 1][r - 1] = table[(r * k) << (LF - 3 - 3 * st)];
+      for (int r = 1; r < 8; ++r) w8[st - 1][r - 1] = table[(r * k) << (LF - 3 - 3 * st)];
+    }
+    if constexpr (TAIL == 2) {
+#pragma unroll
+      for (int r = 1; r < 4; ++r) {
+        wt[r - 1] = table[r * j];
+        wt[r + 2] = table[r * (j + TPL)];
       }
-      if constexpr (TAIL == 2) {
+    } else if constexpr (TAIL == 1) {
 #pragma unroll
-        for (int r = 1; r < 4; ++r) {
-          wt[r - 1] = table[r * j];
-          wt[r + 2] = table[r * (j + TPL)];
-        }
-      } else if constexpr (TAIL == 1) {
-#pragma unroll
-        for (int u = 0; u < 4; ++u) wt[u] = table[j + u * TPL];
-      }
+      for (int u = 0; u < 4; ++u) wt[u] = table[j + u * TPL];
     }
   }
 
@@ -152,20 +151,27 @@ struct ExRow {
   int pstride;      // buffer 1 - buffer 0
   int bar_id;       // named barrier of the line (1 + line in the CTA)
   int bar_n;        // threads of the line
+  void* red;        // lines of several warps: one slot per warp of the CTA for join() (float64)
   __device__ __forceinline__ C* operator()(int par, int m) const { return base + par * pstride + lidx(m); }
+  __device__ __forceinline__ unsigned int addr(int par, int m) const {
+    return (unsigned int)__cvta_generic_to_shared(base) + (unsigned int)sizeof(C) * (unsigned int)(par * pstride + lidx(m));
+  }
   __device__ __forceinline__ void sync() const {
     if (bar_n <= 32) __syncwarp();
     else asm volatile("bar.sync %0, %1;\n" ::"r"(bar_id), "r"(bar_n) : "memory");
   }
-};
-
-// The line symbol: c2 lam^2 + c1 coord lam, lam = dlam * (m or m - F).
-template <typename T, int F>
-struct LineSym {
-  T c2, c1c, dl;
-  __device__ __forceinline__ T operator()(int m) const {
-    const T lm = dl * (T)(m < (F >> 1) ? m : m - F);
-    return (c2 * lm + c1c) * lm;
+  // m joined over the line's threads (consecutive lanes)
+  template <typename M> __device__ __forceinline__ M join(M m) const {
+    for (int o = 1; o < bar_n && o < 32; o <<= 1) m = mag_join(m, mag_shfl_xor(m, o));
+    if (bar_n > 32) {
+      M* r = reinterpret_cast<M*>(red);
+      const int nw = bar_n >> 5, w = (int)threadIdx.x >> 5, w0 = w & ~(nw - 1);
+      if ((threadIdx.x & 31) == 0) r[w] = m;
+      sync();
+      m = r[w0];
+      for (int i = 1; i < nw; ++i) m = mag_join(m, r[w0 + i]);
+    }
+    return m;
   }
 };
 

@@ -28,15 +28,15 @@
 #include <stdlib.h>
 #include "ops_launch.cuh"
 #include "linefft.cuh"
+#include "fixfft.cuh"
 #include "fused2d.cuh"
 
 namespace gpe {
 
 // Threads of the x-kernel's CTA: 256 in float32.  In float64 a CTA holds as
 // few lines as it can (64 threads, or one line of F/8 threads): the float64
-// stages run on small grids (256^2: 16 CTAs of 256 threads), and the float64
-// FMA rate of one SM is 1/64 of its float32 rate, so spreading the lines over
-// more SMs is what shortens them.  At most 128 registers per thread.
+// stages run on small grids (256^2: 16 CTAs of 256 threads), and spreading the
+// lines over more SMs is what shortens them.  At most 128 registers per thread.
 template <typename T> __host__ __device__ constexpr int lines_x_threads(int lf) {
   return sizeof(T) == 4 ? 256 : ((1 << lf) / 8 > 64 ? (1 << lf) / 8 : 64);
 }
@@ -58,17 +58,41 @@ struct ExCols {
     const int ms = m ^ ((m >> 3) & MASK);
     return base + par * pstride + ms * CW;
   }
+  __device__ __forceinline__ unsigned int addr(int par, int m) const {
+    const int ms = m ^ ((m >> 3) & MASK);
+    return (unsigned int)__cvta_generic_to_shared(base) + (unsigned int)sizeof(C) * (unsigned int)(par * pstride + ms * CW);
+  }
+  void* red;        // one slot per warp and column for join() (float64)
   // a column's points are spread over all warps of the CTA
   __device__ __forceinline__ void sync() const { __syncthreads(); }
+  // m joined over the column's threads (every CW-th lane of every warp)
+  template <typename M> __device__ __forceinline__ M join(M m) const {
+#pragma unroll
+    for (int o = CW; o < 32; o <<= 1) m = mag_join(m, mag_shfl_xor(m, o));
+    M* r = reinterpret_cast<M*>(red);
+    const int lane = threadIdx.x & 31, cl = lane & (CW - 1), nw = blockDim.x >> 5;
+    if (lane < CW) r[(threadIdx.x >> 5) * CW + lane] = m;
+    __syncthreads();
+    m = r[cl];
+    for (int i = 1; i < nw; ++i) m = mag_join(m, r[i * CW + cl]);
+    return m;
+  }
 };
 
 
 // Threads of the y-kernel's CTA: 512 in float32 (8 columns of 512 points, 64 B
 // row segments); in float64 as few columns as a line allows, as for the
-// x-kernel.
+// x-kernel, but at least two (32 B segments).
 template <typename T> __host__ __device__ constexpr int lines_y_threads(int lf) {
-  return sizeof(T) == 4 ? 512 : lines_x_threads<T>(lf);
+  return sizeof(T) == 4 ? 512 : ((1 << lf) / 4 > 64 ? (1 << lf) / 4 : 64);
 }
+
+// The twiddle table of a line transform: float32 values, or the halves of
+// 62-bit fractions (float64 grids).
+template <typename FFT>
+__device__ __forceinline__ const typename FFT::Tw* line_table(const PassGeom<float>& G) { return G.tw; }
+template <typename FFT>
+__device__ __forceinline__ const typename FFT::Tw* line_table(const PassGeom<double>& G) { return G.twf; }
 
 // Copy of the twiddle table e^{-2 pi i n / F} into shared memory.
 template <typename C>
@@ -92,11 +116,13 @@ __global__ void __launch_bounds__(lines_y_threads<T>(LF)) k_lines_y(PassGeom<T> 
   constexpr int F = FFT::F;
   if (D.ctl && D.ctl->done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* tws = reinterpret_cast<C*>(smem_raw);
-  C* xb = tws + F;                            // [2][F][CW], swizzled points
-  C* pf0 = xb + 2 * F * CW;                   // [8][NT]: next group's input
+  using X = typename FFT::X;
+  typename FFT::Tw* tws = reinterpret_cast<typename FFT::Tw*>(smem_raw);
+  X* xb = reinterpret_cast<X*>(tws + F);      // [2][F][CW], swizzled points
+  C* pf0 = reinterpret_cast<C*>(xb + 2 * F * CW);   // [8][NT]: next group's input
   C* pf1 = pf0 + 8 * NT;                      // [8][NT]: next group's second operand
-  load_table(tws, G.tw, F);
+  __shared__ long long s_red[(NT / 32) * CW];
+  load_table(tws, line_table<FFT>(G), F);
   const int tid = threadIdx.x;
   const int cl = tid & (CW - 1), j = tid / CW;
   FFT fft;
@@ -122,7 +148,7 @@ __global__ void __launch_bounds__(lines_y_threads<T>(LF)) k_lines_y(PassGeom<T> 
   LineSym<T, F> sym;
   sym.c2 = G.c2;
   sym.dl = G.dlam;
-  ExCols<C, CW> ex{xb + cl, F * CW};
+  ExCols<X, CW> ex{xb + cl, F * CW, s_red};
   auto ebase = [&](int gidx) {
     const int inst = gidx / colgroups;
     const int ccol = (gidx - inst * colgroups) * CW + cl;
@@ -185,12 +211,14 @@ __global__ void __launch_bounds__(lines_x_threads<T>(LF), lines_x_minb<T>(LF)) k
   constexpr int NV = CPLX ? 8 : 16;           // values per thread and group (real: two rows)
   if (D.ctl && D.ctl->done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* tws = reinterpret_cast<C*>(smem_raw);
-  C* xb = tws + F;                            // [2][NL][P]
+  using X = typename FFT::X;
+  typename FFT::Tw* tws = reinterpret_cast<typename FFT::Tw*>(smem_raw);
+  X* xb = reinterpret_cast<X*>(tws + F);      // [2][NL][P]
+  __shared__ long long s_red[NT / 32];
   V* xs = reinterpret_cast<V*>(xb + 2 * NL * FFT::P);   // [2][NV][NT] input, double-buffered
   V* ea = xs + 2 * NV * NT;                   // [NV][NT] T_y X of this group
   T* ev = reinterpret_cast<T*>(ea + NV * NT); // [NV][NT] potential of this group
-  load_table(tws, G.tw, F);
+  load_table(tws, line_table<FFT>(G), F);
   const int tid = threadIdx.x;
   const int l = tid / TPL, j = tid & (TPL - 1);
   FFT fft;
@@ -223,7 +251,7 @@ __global__ void __launch_bounds__(lines_x_threads<T>(LF), lines_x_minb<T>(LF)) k
   // lines of F >= 256 points occupy whole warps (TPL >= 32 threads); the
   // CTA's NL <= 8 lines take named barriers 1..NL
   static_assert(TPL < 32 || (TPL % 32 == 0 && NL <= 15), "named barriers per line");
-  ExRow<C, FFT::P> ex{xb + l * FFT::P, NL * FFT::P, 1 + l, TPL};
+  ExRow<X, FFT::P> ex{xb + l * FFT::P, NL * FFT::P, 1 + l, TPL, s_red};
   // element of value q (q = s, or s + 8 for the second row of a real pair)
   auto gidx = [&](int grp, int q) -> long long {
     const int line = grp * NL + l;

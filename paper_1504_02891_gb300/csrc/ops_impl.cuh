@@ -804,7 +804,8 @@ __device__ __forceinline__ void epilogue_point(const EpiCtx<T, CPLX>& E, long lo
     const V p = ldv<COH>(E.base + gi);
     const T p2 = tre(p, p);
     const T R = tre(p, x);
-    E.out[gi] = lin + E.nl * (p2 * x + (T(2) * R) * p) + E.shift * x;
+    // gathered by x and p: 12 operations a complex point instead of 18 (float64 issues 2 a clock)
+    E.out[gi] = lin + (E.nl * p2 + E.shift) * x + (T(2) * E.nl * R) * p;
   } else if (EPI == EPI_F || EPI == EPI_W) {
     const V y = x;
     V g;

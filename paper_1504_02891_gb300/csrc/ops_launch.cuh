@@ -2,6 +2,7 @@
 // precision by ops_f32.cu / ops_f64.cu.
 #pragma once
 #include <math.h>
+#include <string.h>
 #include <algorithm>
 #include "ops_impl.cuh"
 
@@ -117,12 +118,41 @@ gpe_status GridDev<T>::create(const GridHost& g) {
         const int p = k < F / 2 ? k : k - F;
         hl[k] = (T)(2.0 * M_PI * (double)p / L);
       }
-      GPE_CUDA(cudaMalloc(&tw[a], sizeof(Cx) * F));
-      GPE_CUDA(cudaMemcpy(tw[a], ht.data(), sizeof(Cx) * F, cudaMemcpyHostToDevice));
+      std::vector<Cx> hx(ht);
+      if constexpr (std::is_same<T, double>::value) {
+        // 62-bit fractions in balanced 32-bit halves (fixfft.cuh)
+        static_assert(sizeof(int4) == sizeof(Cx), "two tables of one element size");
+        hx.resize(2 * (size_t)F);
+        const long double one = 4611686018427387904.0L, two_pi = 6.283185307179586476925286766559005768L;
+        std::vector<long long> q(F / 4 + 1);   // a quarter wave of the cosine
+        for (int k = 0; k <= F / 4; ++k) {
+          const int m = std::min(k, F / 4 - k);
+          const long double ang = two_pi * (long double)m / (long double)F;
+          q[k] = llroundl((m == k ? cosl(ang) : sinl(ang)) * one);
+        }
+        auto cosq = [&](int k) -> long long {
+          k &= F - 1;
+          if (k > F / 2) k = F - k;
+          return k <= F / 4 ? q[k] : -q[F / 2 - k];
+        };
+        for (int k = 0; k < F; ++k) {
+          const long long v[2] = {cosq(k), cosq(k + F / 4)};   // cos, -sin of 2 pi k / F
+          int h[4];
+          for (int i = 0; i < 2; ++i) {
+            h[2 * i + 1] = (int)(unsigned int)(v[i] & 0xffffffffLL);
+            if (h[2 * i + 1] == INT32_MIN) h[2 * i + 1] += 1;   // it is negated there; off by 2^-62
+            h[2 * i] = (int)((v[i] - (long long)h[2 * i + 1] + 1) >> 32);
+          }
+          memcpy(&hx[(size_t)F + k], h, sizeof(h));
+        }
+      }
+      GPE_CUDA(cudaMalloc(&tw[a], sizeof(Cx) * hx.size()));
+      GPE_CUDA(cudaMemcpy(tw[a], hx.data(), sizeof(Cx) * hx.size(), cudaMemcpyHostToDevice));
       GPE_CUDA(cudaMalloc(&lam[a], sizeof(T) * F));
       GPE_CUDA(cudaMemcpy(lam[a], hl.data(), sizeof(T) * F, cudaMemcpyHostToDevice));
       PassGeom<T> G = make_geom<T>(a, g.ext, F, F, g.disc == GPE_SINE, g.is_complex, g.nbatch, &blocks[a], &smem[a]);
       G.tw = tw[a];
+      if constexpr (std::is_same<T, double>::value) G.twf = reinterpret_cast<const int4*>(tw[a] + F);
       G.lam = lam[a];
       G.dlam = (T)(2.0 * M_PI / L);
       G.c2 = (T)(0.5 / F);
