@@ -3,6 +3,7 @@
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <stdlib.h>
 #include <string>
 #include <vector>
 #include "gpe_kernels.cuh"
@@ -147,6 +148,22 @@ gpe_status launch_cluster_alg1(ClusterArgs A, int cplx, cudaStream_t st);
 bool cluster_shape(int n0, int n1, int cplx, int nvec, int* cs, int* lch, int* P0, int* P1, size_t* smem,
                    unsigned int* vec_bytes, unsigned int* vpot_bytes, size_t share = 16 * 1024, int* lf = nullptr);
 
+// GPE_LINES2D=0 in the environment selects the general axis-pass kernels
+// instead of the register line kernels (for comparisons); read once.
+static inline bool lines2d_enabled() {
+  static const bool on = [] {
+    const char* e = getenv("GPE_LINES2D");
+    return !(e && e[0] == '0');
+  }();
+  return on;
+}
+
+// The line kernels of the other grids (lines3.cuh): complex and real Fourier
+// lines and real sine lines of 32 to 1024 transform points.
+static inline bool line_axis_ok(const GridHost& g, int a) {
+  if (g.disc == GPE_FD || (g.disc == GPE_SINE && g.is_complex)) return false;
+  return g.F[a] >= 32 && g.F[a] <= 1024 && lines2d_enabled();
+}
 void destroy_solver_cache(void* cache);
 
 // Polls after which a bounded device wait gives up (gpe_set_wait_limit;

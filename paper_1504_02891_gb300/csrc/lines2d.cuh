@@ -25,7 +25,6 @@
 // into the coefficients, the inverse transform taken as a conjugated forward
 // transform.
 #pragma once
-#include <stdlib.h>
 #include "ops_launch.cuh"
 #include "linefft.cuh"
 #include "fixfft.cuh"
@@ -313,8 +312,8 @@ __global__ void __launch_bounds__(lines_x_threads<T>(LF), lines_x_minb<T>(LF)) k
       else kin = (q < 8) ? v[q].x : v[q - 8].y;
       if (accin) kin = kin + ea[q * NT + tid];
       const V lin = kin + ev[q * NT + tid] * x;
-      if constexpr (FPART) epilogue_point<T, CPLX, EPI, false>(E, gi, x, lin, pacc, amax);
-      else epilogue_point<T, CPLX, EPI, false>(E, gi, x, lin, acc, amax);
+      if constexpr (FPART) epilogue_point<T, CPLX, EPI, 2>(E, gi, x, lin, pacc, amax);
+      else epilogue_point<T, CPLX, EPI, 2>(E, gi, x, lin, acc, amax);
     }
     if constexpr (FPART) {
 #pragma unroll
@@ -454,17 +453,6 @@ static gpe_status lines2d_dispatch0(const GridDev<T>& d, const PassData<T>& D, i
     case 10: return lines2d_dispatch1<T, CPLX, EPI, 10>(d, D, nbatch, acc, step_first, lf1, st);
   }
   return fail(GPE_EINVAL, "unsupported line length");
-}
-
-// GPE_LINES2D=0 in the environment selects the general axis-pass kernels
-// instead (for comparisons); read once.
-static bool lines2d_enabled() {
-  static int on = -1;
-  if (on < 0) {
-    const char* e = getenv("GPE_LINES2D");
-    on = (e && e[0] == '0') ? 0 : 1;
-  }
-  return on != 0;
 }
 
 template <typename T>

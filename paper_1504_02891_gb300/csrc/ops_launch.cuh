@@ -90,6 +90,31 @@ static PassGeom<T> make_geom(int axis, const int ext[3], int F, int Fbuf, int od
   return G;
 }
 
+// cos(2 pi k / F), k = 0 .. F/4, as 62-bit fractions (F a power of two >= 4).
+// The points 2^i come from the long double functions, the others are products
+// of two earlier ones in 128-bit integers (a few units of 2^-62; the functions
+// cost 0.7 us a point where long double is emulated, 90 us per plan).
+static inline void quarter_wave_q62(int F, long long* c) {
+  const long double one = 4611686018427387904.0L, two_pi = 6.283185307179586476925286766559005768L;
+  std::vector<long long> s(F / 4 + 1);
+  c[0] = 1LL << 62;
+  s[0] = 0;
+  for (int k = 1; k <= F / 4; ++k) {
+    int p = 1;
+    while (2 * p <= k) p *= 2;
+    const int r = k - p;
+    if (r == 0) {
+      const long double ang = two_pi * (long double)k / (long double)F;
+      c[k] = llroundl(cosl(ang) * one);
+      s[k] = llroundl(sinl(ang) * one);
+    } else {
+      const __int128 h = (__int128)1 << 61;
+      c[k] = (long long)(((__int128)c[p] * c[r] - (__int128)s[p] * s[r] + h) >> 62);
+      s[k] = (long long)(((__int128)s[p] * c[r] + (__int128)c[p] * s[r] + h) >> 62);
+    }
+  }
+}
+
 template <typename T>
 gpe_status GridDev<T>::create(const GridHost& g) {
   using Cx = typename C2t<T>::type;
@@ -123,13 +148,8 @@ gpe_status GridDev<T>::create(const GridHost& g) {
         // 62-bit fractions in balanced 32-bit halves (fixfft.cuh)
         static_assert(sizeof(int4) == sizeof(Cx), "two tables of one element size");
         hx.resize(2 * (size_t)F);
-        const long double one = 4611686018427387904.0L, two_pi = 6.283185307179586476925286766559005768L;
         std::vector<long long> q(F / 4 + 1);   // a quarter wave of the cosine
-        for (int k = 0; k <= F / 4; ++k) {
-          const int m = std::min(k, F / 4 - k);
-          const long double ang = two_pi * (long double)m / (long double)F;
-          q[k] = llroundl((m == k ? cosl(ang) : sinl(ang)) * one);
-        }
+        quarter_wave_q62(F, q.data());
         auto cosq = [&](int k) -> long long {
           k &= F - 1;
           if (k > F / 2) k = F - k;
@@ -409,6 +429,54 @@ gpe_status launch_lines2d(const GridHost& g, const GridDev<T>& d, const PassData
                           bool step_first, cudaStream_t st, bool* handled);
 
 template <typename T>
+gpe_status launch_axis_s(const GridHost& g, const GridDev<T>& d, int axis, const PassData<T>& D, cudaStream_t st);
+template <typename T, int EPI>
+gpe_status launch_axis_x(const GridHost& g, const GridDev<T>& d, const PassData<T>& D, cudaStream_t st);
+
+// Epilogues the x line kernel runs: the float32 solver never runs the model
+// objective W, the float64 one never its difference form.  Float32 gradients
+// keep the general passes: energies of float32 states (and of steps made from
+// such gradients) move in their 7th to 9th digit with the rounding of the
+// transforms, and what callers get for a state stays what it was.
+template <typename T> constexpr bool axis_x_takes(int epi) {
+  return epi == EPI_HESS || epi == EPI_F || epi == EPI_RATIO || epi == (sizeof(T) == 4 ? EPI_WS : EPI_W) ||
+         (epi == EPI_GRAD && sizeof(T) == 8);
+}
+
+// The axes from the last to x, each by its line kernel or, where that does not
+// take the line length, by the general axis pass; x has the epilogue.
+template <typename T>
+gpe_status apply_axes(const GridHost& g, const GridDev<T>& d, const PassData<T>& D, int epi, void* acc, bool step_first,
+                      cudaStream_t st) {
+  for (int a = g.dim - 1; a >= 0; --a) {
+    PassData<T> Da = D;
+    Da.step_on_load = (step_first && a == g.dim - 1) ? 1 : 0;
+    Da.acc_in = a < g.dim - 1 ? acc : nullptr;
+    gpe_status s = GPE_OK;
+    if (a > 0) {
+      Da.out = acc;
+      Da.nq = 0;
+      Da.control = 0;
+      s = line_axis_ok(g, a) ? launch_axis_s<T>(g, d, a, Da, st) : launch_pass<T>(d, a, Da, g.is_complex, EPI_ACC, st);
+    } else if (!line_axis_ok(g, a)) {
+      s = launch_pass<T>(d, a, Da, g.is_complex, epi, st);
+    } else {
+      switch (epi) {
+        case EPI_GRAD:
+          if constexpr (axis_x_takes<T>(EPI_GRAD)) s = launch_axis_x<T, EPI_GRAD>(g, d, Da, st);
+          break;
+        case EPI_HESS: s = launch_axis_x<T, EPI_HESS>(g, d, Da, st); break;
+        case EPI_F: s = launch_axis_x<T, EPI_F>(g, d, Da, st); break;
+        case EPI_RATIO: s = launch_axis_x<T, EPI_RATIO>(g, d, Da, st); break;
+        default: s = launch_axis_x<T, sizeof(T) == 4 ? EPI_WS : EPI_W>(g, d, Da, st); break;
+      }
+    }
+    if (s != GPE_OK) return s;
+  }
+  return GPE_OK;
+}
+
+template <typename T>
 gpe_status apply_op(const GridHost& g, const GridDev<T>& d, PassData<T> D, int epi, void* acc, bool step_first,
                     cudaStream_t st) {
   if (g.disc == GPE_FOURIER && g.dim == 2) {
@@ -423,6 +491,9 @@ gpe_status apply_op(const GridHost& g, const GridDev<T>& d, PassData<T> D, int e
     }
     return launch_fd<T>(d, D, g.is_complex, epi, st);
   }
+  if (axis_x_takes<T>(epi))
+    for (int a = 0; a < g.dim; ++a)
+      if (line_axis_ok(g, a)) return apply_axes<T>(g, d, D, epi, acc, step_first, st);
   for (int a = 0; a < g.dim; ++a) {
     PassData<T> Da = D;
     Da.step_on_load = (step_first && a == 0) ? 1 : 0;

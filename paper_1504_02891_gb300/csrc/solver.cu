@@ -338,7 +338,12 @@ static gpe_status alg1_run(Level<T>& L, int objective, int first_slot, int max_i
   long long launched = 0;
   s = read_ctl<T>(L, st);
   if (s != GPE_OK) return s;
-  if (!L.h_ctl->done && P.persistent && objective < 2 && !prof_enabled()) {
+  // 3D grids that the line kernels take run faster as queued chunks of them
+  // than as one persistent launch of general pass tiles (64^3 sine float32: 16
+  // against 60 us an iteration)
+  bool queued = L.g.dim == 3;
+  for (int a = 0; a < L.g.dim; ++a) queued = queued && line_axis_ok(L.g, a);
+  if (!L.h_ctl->done && P.persistent && !queued && objective < 2 && !prof_enabled()) {
     if (L.p_grid[objective] < 0) {
       s = persist_config<T>(L.g, L.d, objective == 1 ? EPI_W : EPI_F, &L.p_grid[objective], &L.p_smem[objective]);
       if (s != GPE_OK) return s;
