@@ -162,7 +162,7 @@ struct FusedSym {
 struct FusedArgs {
   void* ty;                 // T_y of the y-tasks (the output array when every point is written)
   unsigned int* sync;       // [0] tasks handed out, [1] warps done, [2, 2+nb) y-tasks done,
-                            // [2+nb, 2+2nb) x-tasks done, [2+2nb] error flag
+                            // [2+nb, 2+2nb) x-tasks done
   int nbatch, NY, NX;       // instances, y-tasks and x-tasks per instance
   long long max_polls;      // polls of one task wait before it gives up
   int skew;                 // instances whose y-tasks precede the first x-task
@@ -332,7 +332,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, fused_minb(LF)) k_fused2d(PassG
         long long polls = 0;
         while (ld_acquire_u32(ydone + b) < (unsigned)NY) {
           if (++polls > FA.max_polls) {
-            atomicExch(cnt + 2 + 2 * nb, 1u);
+            if (D.err) *D.err = 1.0;
             ok = 0;
             break;
           }
@@ -500,7 +500,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, fused_minb(LF)) k_fused2d(PassG
     }
   }
   // the last warp to finish resets the counters for the next launch (every
-  // warp has stopped taking tasks by then); the error flag stays set
+  // warp has stopped taking tasks by then)
   __syncwarp();
   int lastw = 0;
   if (lane == 0) lastw = atom_add_acqrel_u32(cnt + 1, 1u) == gridDim.x * (blockDim.x >> 5) - 1;

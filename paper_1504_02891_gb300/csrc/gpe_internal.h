@@ -77,7 +77,7 @@ struct GridDev {
   // 2D Fourier grids (fused warp-line kernel, fused2d.cuh): per axis the
   // twiddles e^{-2 pi i j k2 / F} in k2-major order (entry k2 * TPL + j, TPL
   // the threads per line), and the launch's counters: task counter, exited
-  // warps, per-instance finished y- and x-tasks, error flag (zero between
+  // warps, per-instance finished y- and x-tasks (zero between
   // launches; the last warp of a launch resets them)
   C* tw2[2] = {nullptr, nullptr};
   unsigned int* fsync = nullptr;
@@ -90,13 +90,18 @@ struct Scratch {
   double* partials = nullptr;
   double* results = nullptr;     // [nbatch][NQ]
   double* coef = nullptr;        // [nbatch][4]
-  unsigned int* ticket = nullptr;
-  double* h_results = nullptr;   // pinned mirror
+  unsigned int* ticket = nullptr;   // [nbatch], zero between launches
+  // [nbatch][NQ] in pinned host memory: the energy entry points have the
+  // reductions write their sums here (no copy to wait for), and the fused
+  // kernel's expired-wait flag behind them
+  double* h_results = nullptr;
   size_t cap_blocks = 0;
   int nbatch = 0;
   gpe_status create(size_t blocks, int nbatch);
   void destroy();
 };
+
+struct MomentCoef;   // ops_impl.cuh: what k_moments makes of its sums
 
 // Launch wrappers (explicitly instantiated for float and double).
 template <typename T>
@@ -108,7 +113,7 @@ gpe_status launch_step(void* const* xs, void* const* gs, const Alg1Ctl* ctl, lon
                        const void* xk = nullptr);
 template <typename T>
 gpe_status launch_moments(const void* x, const void* g, long long M, int nbatch, int cplx, Scratch& sc,
-                          cudaStream_t st);
+                          const MomentCoef& mc, cudaStream_t st);
 template <typename T>
 gpe_status launch_axpby(const void* x, const void* g, const double* coef, int stride_coef, long long M, int nbatch,
                         void* out, int cplx, cudaStream_t st);
@@ -119,8 +124,6 @@ gpe_status launch_prolong(const GridHost& gc, const GridHost& gf, const GridDev<
                           const void* in, void* out, void* tmp1, void* tmp2, cudaStream_t st);
 template <typename Ti, typename To>
 gpe_status launch_convert(const Ti* in, To* out, long long n, double scale, cudaStream_t st);
-gpe_status launch_step_coef(const double* mom, int nbatch, double h, double tau, double* coef, cudaStream_t st);
-gpe_status launch_norm_coef(const double* mom, int nbatch, double h, double* coef, cudaStream_t st);
 gpe_status launch_to_shifted_f32(const double* xk, const double* gk, double th, float* xk32, float* pk32, long long n,
                                  cudaStream_t st);
 gpe_status launch_add_f32_to_f64(const double* xk, const float* d, double* z, long long n, cudaStream_t st);

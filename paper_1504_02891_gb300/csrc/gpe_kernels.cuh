@@ -210,7 +210,8 @@ struct PassData {
   // reductions
   double* partials;     // [gridDim.x][NQ]
   double* results;      // [nbatch][NQ]
-  unsigned int* ticket;
+  unsigned int* ticket; // [nbatch]
+  double* err;          // fused kernel: set to 1 when a task wait gave up (may be null)
   int nq;               // active slots (0: none)
   int control;          // 0: none, 1: Algorithm 1 control, 2: ratio control
 };

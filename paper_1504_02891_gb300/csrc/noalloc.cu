@@ -33,7 +33,7 @@ constexpr size_t NOALLOC_BYTES = 512 * 1024;
 static_assert((NOALLOC_PARTIALS + NOALLOC_RESULTS + NOALLOC_COEF) * sizeof(double) + 256 <= NOALLOC_BYTES,
               "scratch layout exceeds the array");
 
-// partials | results | coef | ticket (unsigned int), each 256-byte aligned
+// partials | results | coef | tickets (unsigned int per instance), each 256-byte aligned
 static __device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_BYTES];
 
 std::mutex g_mu;
@@ -111,14 +111,12 @@ gpe_status run(const void* psi, const void* hpsi, long long M, int nbatch, doubl
   double* results = partials + NOALLOC_PARTIALS;
   double* coef = results + NOALLOC_RESULTS;
   unsigned int* ticket = reinterpret_cast<unsigned int*>(coef + NOALLOC_COEF);
-  // the array keeps the previous call's contents: the ticket must start at zero
-  cudaError_t e = cudaMemsetAsync(ticket, 0, sizeof(unsigned int), st);
+  // the array keeps the previous call's contents: the tickets must start at zero
+  cudaError_t e = cudaMemsetAsync(ticket, 0, sizeof(unsigned int) * NOALLOC_MAX_BATCH, st);
   if (e != cudaSuccess) return gpe::cuda_fail(e, "cudaMemsetAsync(ticket)");
-  gpe::k_moments<T, CPLX><<<tiles * nbatch, gpe::NTHREADS, 0, st>>>(psi, hpsi, M, tiles, partials, results, ticket);
-  gpe::k_step_coef<<<(nbatch + 127) / 128, 128, 0, st>>>(results, nbatch, h, tau, coef);
-  const long long n = M * nbatch;
-  const int eb = (int)std::max<long long>(1, std::min<long long>((n + gpe::NTHREADS - 1) / gpe::NTHREADS, 152 * 8));
-  gpe::k_axpby<T, CPLX><<<eb, gpe::NTHREADS, 0, st>>>(psi, hpsi, coef, 2, M, nbatch, out);
+  const gpe::MomentCoef mc{1, h, tau, coef};
+  gpe::run_moments<T, CPLX>(psi, hpsi, M, nbatch, tiles, partials, results, ticket, mc, st);
+  gpe::run_axpby<T, CPLX>(psi, hpsi, coef, 2, M, nbatch, out, st);
   e = cudaGetLastError();
   if (e != cudaSuccess) return gpe::cuda_fail(e, "gpe_feasible_step_noalloc launch");
   return GPE_OK;

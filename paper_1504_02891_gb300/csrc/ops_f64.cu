@@ -17,19 +17,6 @@ template gpe_status launch_convert<double, float>(const double*, float*, long lo
 template gpe_status launch_convert<float, float>(const float*, float*, long long, double, cudaStream_t);
 template gpe_status launch_convert<double, double>(const double*, double*, long long, double, cudaStream_t);
 
-gpe_status launch_step_coef(const double* mom, int nbatch, double h, double tau, double* coef, cudaStream_t st) {
-  ProfScope ps("step_coef", st);
-  k_step_coef<<<(nbatch + 127) / 128, 128, 0, st>>>(mom, nbatch, h, tau, coef);
-  GPE_CUDA(cudaGetLastError());
-  return GPE_OK;
-}
-
-gpe_status launch_norm_coef(const double* mom, int nbatch, double h, double* coef, cudaStream_t st) {
-  ProfScope ps("norm_coef", st);
-  k_norm_coef<<<(nbatch + 127) / 128, 128, 0, st>>>(mom, nbatch, h, coef);
-  GPE_CUDA(cudaGetLastError());
-  return GPE_OK;
-}
 }  // namespace gpe
 
 namespace gpe {

@@ -2,6 +2,8 @@
 // ops_f32.cu and ops_f64.cu.  See gpe_kernels.cuh for the design summary.
 #pragma once
 #include <math.h>
+#include <stdint.h>
+#include <algorithm>
 #include <type_traits>
 #include "gpe_kernels.cuh"
 #include "gpe_internal.h"
@@ -462,68 +464,24 @@ static __device__ void fold_partials(const double* partials, int tiles, int nq, 
   __syncthreads();
 }
 
-// Several instances: warp w folds instances w, w + nwarps, ... (lanes stride
-// over the tiles in a fixed order, then a fixed shuffle tree), so the final
-// fold of a large batch is spread over the CTA's warps.  Ends with a barrier.
-template <typename A>
-static __device__ void fold_partials_warps(const double* partials, int tiles, int nq, double* results, int ninst) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int nw = blockDim.x >> 5;
-  const A* pp = reinterpret_cast<const A*>(partials);
-  for (int b = warp; b < ninst; b += nw) {
-    for (int q = 0; q < NQ; ++q) {
-      if (q >= nq && q != Q_MAX) {
-        if (lane == 0) results[(size_t)b * NQ + q] = 0.0;
-        continue;
-      }
-      A x;
-      acc_zero(x);
-      for (int i = lane; i < tiles; i += 32) {
-        const size_t o = ((size_t)b * tiles + i) * NQ + q;
-        if constexpr (std::is_same<A, double>::value) {
-          const double w = __ldcg(pp + o);
-          x = (q == Q_MAX) ? fmax(x, w) : x + w;
-        } else {
-          const float2 f = __ldcg(reinterpret_cast<const float2*>(pp + o));
-          A w;
-          w.hi = f.x;
-          w.lo = f.y;
-          if (q == Q_MAX) df_max(x, w);
-          else acc_merge(x, w);
-        }
-      }
-      for (int o = 16; o > 0; o >>= 1) {
-        if constexpr (std::is_same<A, double>::value) {
-          const double w = __shfl_down_sync(0xffffffffu, x, o);
-          x = (q == Q_MAX) ? fmax(x, w) : x + w;
-        } else {
-          const DF w = shfl_down(x, o);
-          if (q == Q_MAX) df_max(x, w);
-          else acc_merge(x, w);
-        }
-      }
-      if (lane == 0) results[(size_t)b * NQ + q] = acc_value(x);
-    }
-  }
-  __syncthreads();
-}
-
-// Block partial, then the last CTA to finish (atomic ticket) folds all
-// partials per instance into results[inst][q].  Returns true in the last CTA.
+// Block partial, then the last CTA of the instance to finish (its own atomic
+// ticket) folds the instance's partials into results[inst][q].  Returns true in
+// that CTA.  One last CTA for the whole batch folded the instances one after
+// another, about 0.5 us for each sum: 64 us of the 82 us of a moments launch
+// over 128 instances.
 template <typename A, typename M>
 static __device__ bool reduce_partials(A (&acc)[NQ], M amax2, int nq, double* partials, double* results,
                                        unsigned int* ticket, int tiles_per_inst) {
   __shared__ int s_last;
+  const int inst = blockIdx.x / tiles_per_inst;
   block_partial(acc, amax2, nq, partials + (size_t)blockIdx.x * NQ);
   __threadfence();
-  if (threadIdx.x == 0) s_last = (atomicAdd(ticket, 1u) == gridDim.x - 1);
+  if (threadIdx.x == 0) s_last = (atomicAdd(ticket + inst, 1u) == (unsigned)tiles_per_inst - 1u);
   __syncthreads();
   if (!s_last) return false;
   __threadfence();
-  const int ninst = gridDim.x / tiles_per_inst;
-  if (ninst == 1) fold_partials<A>(partials, tiles_per_inst, nq, results);
-  else fold_partials_warps<A>(partials, tiles_per_inst, nq, results, ninst);
-  if (threadIdx.x == 0) *ticket = 0u;
+  fold_partials<A>(partials + (size_t)inst * tiles_per_inst * NQ, tiles_per_inst, nq, results + (size_t)inst * NQ);
+  if (threadIdx.x == 0) ticket[inst] = 0u;
   __threadfence();
   __syncthreads();
   return true;
@@ -1314,74 +1272,155 @@ __global__ void k_step(void* const* xs, void* const* gs, const Alg1Ctl* c, long 
     Y[i] = a * X[i] + b * Gv[i];
 }
 
-// Per-instance sums |x|^2, Re conj(x) g, |g|^2 (g may be null).
-template <typename T, bool CPLX>
+// What the last CTA of an instance makes of its moments: nothing, the Cayley
+// coefficients of gpe_feasible_step (grid units in, unified units inside:
+// X = sqrt(h) psi, G = 2 sqrt(h) hpsi), or the scale to unit discrete norm.
+struct MomentCoef {
+  int mode;        // 0: none, 1: step, 2: norm
+  double h, tau;
+  double* coef;    // [nbatch][2] (step) or [nbatch] (norm)
+};
+static __device__ void moment_coef(const MomentCoef& mc, int b, const double* r) {
+  if (mc.mode == 1) {
+    const double h = mc.h;
+    const double nX = h * r[0], XG = 2.0 * h * r[1], GG = 4.0 * h * r[2];
+    double PP = GG - XG * XG / nX;
+    if (PP < 0.0) PP = 0.0;
+    const double t = mc.tau, nxpp = nX * PP, den = 1.0 + t * t * nxpp;
+    const double a = (1.0 + 2.0 * t * XG - t * t * nxpp) / den;
+    const double bb = -2.0 * t * nX / den;
+    const double ny = a * a * nX + 2.0 * a * bb * XG + bb * bb * GG;
+    const double s = 1.0 / sqrt(ny);
+    // psi_out = (s a X + s b G) / sqrt(h) = s a psi + 2 s b hpsi
+    mc.coef[(size_t)b * 2 + 0] = s * a;
+    mc.coef[(size_t)b * 2 + 1] = 2.0 * s * bb;
+  } else if (mc.mode == 2) {
+    mc.coef[b] = 1.0 / sqrt(mc.h * r[0]);
+  }
+}
+
+// Re(conj(a) b) of the moments with a fixed rounding, whatever the compiler
+// would contract: the step's float32 coefficients depend on it.
+__device__ __forceinline__ float mre(float a, float b) { return a * b; }
+__device__ __forceinline__ double mre(double a, double b) { return a * b; }
+__device__ __forceinline__ float mre(float2 a, float2 b) { return __fmaf_rn(a.x, b.x, __fmul_rn(a.y, b.y)); }
+__device__ __forceinline__ double mre(double2 a, double2 b) { return a.x * b.x + a.y * b.y; }
+
+// Several values of a field as one 16-byte access (field arrays that start on
+// 16 bytes for every instance), or one value.
+template <typename V, int W> struct alignas(sizeof(V) * W) Pack {
+  V v[W];
+};
+
+// Per-instance sums |x|^2, Re conj(x) g, |g|^2 (g may be null), W values per
+// access.  A few CTAs per SM stride over their instance: with one value per
+// thread the block reductions cost several times the reading.  128 x 128^2
+// complex64: 82 us with one value per thread and one fold for the batch.
+template <typename T, bool CPLX, int W>
 __global__ void __launch_bounds__(NTHREADS) k_moments(const void* xv, const void* gv, long long M, int tiles,
-                                                      double* partials, double* results, unsigned int* ticket) {
+                                                      double* partials, double* results, unsigned int* ticket,
+                                                      MomentCoef mc) {
   using V = typename VT<T, CPLX>::V;
-  const V* x = (const V*)xv;
-  const V* g = (const V*)gv;
+  using P = Pack<V, W>;
   const int inst = blockIdx.x / tiles;
   const int tb = blockIdx.x - inst * tiles;
+  const P* x = reinterpret_cast<const P*>((const V*)xv + inst * M);
+  const P* g = gv ? reinterpret_cast<const P*>((const V*)gv + inst * M) : nullptr;
   using A = typename AccT<T>::type;
   A acc[NQ];
 #pragma unroll
   for (int q = 0; q < NQ; ++q) acc_zero(acc[q]);
-  const long long base = inst * M;
-  for (long long i = (long long)tb * blockDim.x + threadIdx.x; i < M; i += (long long)tiles * blockDim.x) {
-    const V xi = x[base + i];
-    acc_add(acc[0], tre(xi, xi));
-    if (g) {
-      const V gi = g[base + i];
-      acc_add(acc[1], tre(xi, gi));
-      acc_add(acc[2], tre(gi, gi));
+  const long long n = M / W;
+#pragma unroll 4
+  for (long long i = (long long)tb * blockDim.x + threadIdx.x; i < n; i += (long long)tiles * blockDim.x) {
+    const P xi = x[i];
+    P gi;
+    if (g) gi = g[i];
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+      acc_add(acc[0], mre(xi.v[w], xi.v[w]));
+      if (g) {
+        acc_add(acc[1], mre(xi.v[w], gi.v[w]));
+        acc_add(acc[2], mre(gi.v[w], gi.v[w]));
+      }
     }
   }
-  reduce_partials(acc, T(0), 3, partials, results, ticket, tiles);
+  if (reduce_partials(acc, T(0), 3, partials, results, ticket, tiles) && threadIdx.x == 0)
+    moment_coef(mc, inst, results + (size_t)inst * NQ);
 }
 
-// out_b = ca[b] * x_b + cb[b] * g_b  (g may be null)
-template <typename T, bool CPLX>
-__global__ void k_axpby(const void* xv, const void* gv, const double* coef, int stride_coef, long long M,
-                        int nbatch, void* outv) {
+// s a and s a + c with one rounding per operation whatever the compiler would
+// contract: the float32 energy of a step depends on them in its 8th digit.
+__device__ __forceinline__ float scaled(float s, float a) { return __fmul_rn(s, a); }
+__device__ __forceinline__ double scaled(double s, double a) { return __dmul_rn(s, a); }
+__device__ __forceinline__ float fused_add(float s, float a, float c) { return __fmaf_rn(s, a, c); }
+__device__ __forceinline__ double fused_add(double s, double a, double c) { return __fma_rn(s, a, c); }
+template <typename T, typename C> __device__ __forceinline__ C scaled(T s, C a) {
+  a.x = scaled(s, a.x);
+  a.y = scaled(s, a.y);
+  return a;
+}
+template <typename T, typename C> __device__ __forceinline__ C fused_add(T s, C a, C c) {
+  c.x = fused_add(s, a.x, c.x);
+  c.y = fused_add(s, a.y, c.y);
+  return c;
+}
+
+// out_b = ca[b] * x_b + cb[b] * g_b  (g may be null), W values per access; the
+// CTAs of row blockIdx.y take the instances y, y + gridDim.y, ...
+template <typename T, bool CPLX, int W>
+__global__ void __launch_bounds__(NTHREADS) k_axpby(const void* xv, const void* gv, const double* coef,
+                                                    int stride_coef, long long M, int nbatch, void* outv) {
   using V = typename VT<T, CPLX>::V;
-  const V* x = (const V*)xv;
-  const V* g = (const V*)gv;
-  V* out = (V*)outv;
-  const long long n = M * nbatch;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const int b = (int)(i / M);
-    const T ca = (T)coef[(size_t)b * stride_coef + 0];
-    V v = ca * x[i];
-    if (g) v = v + (T)coef[(size_t)b * stride_coef + 1] * g[i];
-    out[i] = v;
+  using P = Pack<V, W>;
+  const long long n = M / W;
+  for (int b = blockIdx.y; b < nbatch; b += gridDim.y) {
+    const P* x = reinterpret_cast<const P*>((const V*)xv + b * M);
+    const P* g = gv ? reinterpret_cast<const P*>((const V*)gv + b * M) : nullptr;
+    P* out = reinterpret_cast<P*>((V*)outv + b * M);
+    const T ca = (T)coef[(size_t)b * stride_coef];
+    const T cb = g ? (T)coef[(size_t)b * stride_coef + 1] : T(0);
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+      const P xi = x[i];
+      P r, gi;
+      if (g) gi = g[i];
+#pragma unroll
+      for (int w = 0; w < W; ++w) {
+        r.v[w] = g ? fused_add(ca, xi.v[w], scaled(cb, gi.v[w])) : scaled(ca, xi.v[w]);
+      }
+      out[i] = r;
+    }
   }
 }
 
-// Coefficients for gpe_feasible_step from the moments (grid units in, unified
-// units inside): X = sqrt(h) psi, G = 2 sqrt(h) hpsi.
-static __global__ void k_step_coef(const double* mom, int nbatch, double h, double tau, double* coef) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= nbatch) return;
-  const double* r = mom + (size_t)b * NQ;
-  const double nX = h * r[0], XG = 2.0 * h * r[1], GG = 4.0 * h * r[2];
-  double PP = GG - XG * XG / nX;
-  if (PP < 0.0) PP = 0.0;
-  const double t = tau, nxpp = nX * PP, den = 1.0 + t * t * nxpp;
-  const double a = (1.0 + 2.0 * t * XG - t * t * nxpp) / den;
-  const double bb = -2.0 * t * nX / den;
-  const double ny = a * a * nX + 2.0 * a * bb * XG + bb * bb * GG;
-  const double s = 1.0 / sqrt(ny);
-  // psi_out = (s a X + s b G) / sqrt(h) = s a psi + 2 s b hpsi
-  coef[(size_t)b * 2 + 0] = s * a;
-  coef[(size_t)b * 2 + 1] = 2.0 * s * bb;
+// Values per 16-byte access, 1 if an instance does not start on 16 bytes.
+static inline int pack_width(size_t vsz, long long M, const void* a, const void* b, const void* c) {
+  const int w = (int)(16 / vsz);
+  const uintptr_t bits = (uintptr_t)a | (uintptr_t)b | (uintptr_t)c;
+  return (w > 1 && M % w == 0 && (bits & 15) == 0) ? w : 1;
 }
-
-// scale to unit discrete norm: coef[b] = 1/sqrt(h * sum|x|^2)
-static __global__ void k_norm_coef(const double* mom, int nbatch, double h, double* coef) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= nbatch) return;
-  coef[b] = 1.0 / sqrt(h * mom[(size_t)b * NQ + 0]);
+template <typename T, bool CPLX>
+static void run_moments(const void* x, const void* g, long long M, int nbatch, int tiles, double* partials,
+                        double* results, unsigned int* ticket, const MomentCoef& mc, cudaStream_t st) {
+  using V = typename VT<T, CPLX>::V;
+  constexpr int W = (int)(16 / sizeof(V));
+  if (pack_width(sizeof(V), M, x, g, nullptr) > 1)
+    k_moments<T, CPLX, W><<<tiles * nbatch, NTHREADS, 0, st>>>(x, g, M, tiles, partials, results, ticket, mc);
+  else
+    k_moments<T, CPLX, 1><<<tiles * nbatch, NTHREADS, 0, st>>>(x, g, M, tiles, partials, results, ticket, mc);
+}
+template <typename T, bool CPLX>
+static void run_axpby(const void* x, const void* g, const double* coef, int stride, long long M, int nbatch, void* out,
+                      cudaStream_t st) {
+  using V = typename VT<T, CPLX>::V;
+  constexpr int W = (int)(16 / sizeof(V));
+  const int w = pack_width(sizeof(V), M, x, g, out);
+  // about eight CTAs per SM in all, one value (pack) per thread and pass
+  const int gy = std::min(nbatch, 65535);
+  const long long full = (M / w + NTHREADS - 1) / NTHREADS;
+  const int gx = (int)std::max<long long>(1, std::min<long long>(full, std::max(1, 152 * 8 / gy)));
+  if (w > 1) k_axpby<T, CPLX, W><<<dim3(gx, gy), NTHREADS, 0, st>>>(x, g, coef, stride, M, nbatch, out);
+  else k_axpby<T, CPLX, 1><<<dim3(gx, gy), NTHREADS, 0, st>>>(x, g, coef, stride, M, nbatch, out);
 }
 
 // Shifted subproblem inputs in float32: X^k and P_k = G_k - theta_k X^k

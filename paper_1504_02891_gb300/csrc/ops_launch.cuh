@@ -206,7 +206,7 @@ gpe_status GridDev<T>::create(const GridHost& g) {
         const int lpw = 32 / fused_tpl(g.ext[0]);
         max_blocks = std::max(max_blocks, std::max(1, lines / lpw) * g.nbatch);
       }
-      const size_t nsync = 3 + 2 * (size_t)g.nbatch;
+      const size_t nsync = 2 + 2 * (size_t)g.nbatch;
       GPE_CUDA(cudaMalloc(&fsync, sizeof(unsigned int) * nsync));
       GPE_CUDA(cudaMemset(fsync, 0, sizeof(unsigned int) * nsync));
     }
@@ -334,12 +334,15 @@ gpe_status launch_step(void* const* xs, void* const* gs, const Alg1Ctl* ctl, lon
 
 template <typename T>
 gpe_status launch_moments(const void* x, const void* g, long long M, int nbatch, int cplx, Scratch& sc,
-                          cudaStream_t st) {
-  const int tiles = (int)std::max<long long>(1, std::min<long long>((M + NTHREADS - 1) / NTHREADS, 512));
+                          const MomentCoef& mc, cudaStream_t st) {
+  // about four CTAs per SM in all, at least four values per thread
+  const long long full = (M + 4 * NTHREADS - 1) / (4 * NTHREADS);
+  const long long most = std::min<long long>(4 * 152 / nbatch, (long long)(sc.cap_blocks / nbatch));
+  const int tiles = (int)std::max<long long>(1, std::min(full, most));
   if ((size_t)tiles * nbatch > sc.cap_blocks) return fail(GPE_EINVAL, "reduction scratch too small");
   ProfScope ps(kernel_name("moments", sizeof(T) == 8, cplx, -1), st);
-  if (cplx) k_moments<T, true><<<tiles * nbatch, NTHREADS, 0, st>>>(x, g, M, tiles, sc.partials, sc.results, sc.ticket);
-  else k_moments<T, false><<<tiles * nbatch, NTHREADS, 0, st>>>(x, g, M, tiles, sc.partials, sc.results, sc.ticket);
+  if (cplx) run_moments<T, true>(x, g, M, nbatch, tiles, sc.partials, sc.results, sc.ticket, mc, st);
+  else run_moments<T, false>(x, g, M, nbatch, tiles, sc.partials, sc.results, sc.ticket, mc, st);
   GPE_CUDA(cudaGetLastError());
   return GPE_OK;
 }
@@ -347,10 +350,9 @@ gpe_status launch_moments(const void* x, const void* g, long long M, int nbatch,
 template <typename T>
 gpe_status launch_axpby(const void* x, const void* g, const double* coef, int stride_coef, long long M, int nbatch,
                         void* out, int cplx, cudaStream_t st) {
-  const long long n = M * nbatch;
   ProfScope ps(kernel_name("axpby", sizeof(T) == 8, cplx, -1), st);
-  if (cplx) k_axpby<T, true><<<ew_blocks(n), NTHREADS, 0, st>>>(x, g, coef, stride_coef, M, nbatch, out);
-  else k_axpby<T, false><<<ew_blocks(n), NTHREADS, 0, st>>>(x, g, coef, stride_coef, M, nbatch, out);
+  if (cplx) run_axpby<T, true>(x, g, coef, stride_coef, M, nbatch, out, st);
+  else run_axpby<T, false>(x, g, coef, stride_coef, M, nbatch, out, st);
   GPE_CUDA(cudaGetLastError());
   return GPE_OK;
 }
@@ -588,7 +590,8 @@ gpe_status launch_alg1_persist(const GridHost& g, const GridDev<T>& d, const Pas
   template gpe_status launch_fd<T>(const GridDev<T>&, const PassData<T>&, int, int, cudaStream_t);                  \
   template gpe_status launch_step<T>(void* const*, void* const*, const Alg1Ctl*, long long, int, cudaStream_t,      \
                                      const void*);                                                                 \
-  template gpe_status launch_moments<T>(const void*, const void*, long long, int, int, Scratch&, cudaStream_t);     \
+  template gpe_status launch_moments<T>(const void*, const void*, long long, int, int, Scratch&, const MomentCoef&, \
+                                        cudaStream_t);                                                             \
   template gpe_status launch_axpby<T>(const void*, const void*, const double*, int, long long, int, void*, int,     \
                                       cudaStream_t);                                                               \
   template gpe_status launch_inject<T>(const GridHost&, const GridHost&, const void*, void*, cudaStream_t);         \

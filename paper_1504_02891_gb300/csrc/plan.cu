@@ -6,7 +6,7 @@
 #include <map>
 #include <mutex>
 #include <string>
-#include "gpe_internal.h"
+#include "ops_impl.cuh"
 
 namespace gpe {
 
@@ -64,6 +64,7 @@ ProfScope::~ProfScope() {
 }
 
 const char* kernel_name(const char* base, int f64, int cplx, int epi, long long points) {
+  if (!prof_enabled()) return base;   // the name is only used by the records
   static const char* epis[] = {"acc", "grad", "hess", "F", "W", "ratio", "WS"};
   static std::mutex mu;
   static std::map<std::string, std::string> names;
@@ -204,10 +205,11 @@ gpe_status Scratch::create(size_t blocks, int nb) {
   GPE_CUDA(cudaMalloc(&partials, sizeof(double) * NQ * blocks));
   GPE_CUDA(cudaMalloc(&results, sizeof(double) * NQ * nb));
   GPE_CUDA(cudaMalloc(&coef, sizeof(double) * 4 * nb));
-  GPE_CUDA(cudaMalloc(&ticket, sizeof(unsigned int)));
-  GPE_CUDA(cudaMemset(ticket, 0, sizeof(unsigned int)));
+  GPE_CUDA(cudaMalloc(&ticket, sizeof(unsigned int) * nb));
+  GPE_CUDA(cudaMemset(ticket, 0, sizeof(unsigned int) * nb));
   GPE_CUDA(cudaMemset(results, 0, sizeof(double) * NQ * nb));
-  GPE_CUDA(cudaMallocHost(&h_results, sizeof(double) * NQ * nb));
+  GPE_CUDA(cudaMallocHost(&h_results, sizeof(double) * ((size_t)NQ * nb + 1)));
+  h_results[(size_t)NQ * nb] = 0.0;
   return GPE_OK;
 }
 
@@ -292,27 +294,24 @@ static PassData<T> abi_data(gpe_plan p, const GridDev<T>& d) {
   D.nl = p->g.beta;
   D.lin_scale = 1.0;
   D.partials = p->sc.partials;
-  D.results = p->sc.results;
+  D.results = p->sc.h_results;
   D.ticket = p->sc.ticket;
+  D.err = p->sc.h_results + (size_t)NQ * p->g.nbatch;
   return D;
 }
 
 // E, mu, norm2 from the GRAD-epilogue sums of each instance.
 static gpe_status read_energy(gpe_plan p, double* E, double* mu, double* norm2) {
   const int nb = p->g.nbatch;
-  GPE_CUDA(cudaMemcpyAsync(p->sc.h_results, p->sc.results, sizeof(double) * NQ * nb, cudaMemcpyDeviceToHost, p->stream));
+  // the reductions have written the sums into pinned host memory
   GPE_CUDA(cudaStreamSynchronize(p->stream));
   gpe_status st = GPE_OK;
   // a bounded task wait of the fused 2D kernel that gave up leaves its flag set
   // (and NaN partial sums): report it as the expired wait it was, then clear it
-  unsigned int* fs = p->prec == GPE_F32 ? p->d32->fsync : p->d64->fsync;
-  if (fs) {
-    unsigned int flag = 0;
-    GPE_CUDA(cudaMemcpy(&flag, fs + 2 + 2 * (size_t)nb, sizeof(flag), cudaMemcpyDeviceToHost));
-    if (flag) {
-      GPE_CUDA(cudaMemset(fs + 2 + 2 * (size_t)nb, 0, sizeof(flag)));
-      return fail(GPE_ETIMEOUT, "a bounded task wait of the fused 2D operator kernel expired");
-    }
+  double& flag = p->sc.h_results[(size_t)NQ * nb];
+  if (flag != 0.0) {
+    flag = 0.0;
+    return fail(GPE_ETIMEOUT, "a bounded task wait of the fused 2D operator kernel expired");
   }
   for (int b = 0; b < nb; ++b) {
     const double* r = p->sc.h_results + (size_t)b * NQ;
@@ -327,17 +326,18 @@ static gpe_status read_energy(gpe_plan p, double* E, double* mu, double* norm2) 
 }
 
 template <typename T>
-static gpe_status do_grad(gpe_plan p, const GridDev<T>& d, const void* psi, void* hpsi) {
+static gpe_status do_grad(gpe_plan p, const GridDev<T>& d, const void* psi, void* hpsi, bool sums) {
   PassData<T> D = abi_data<T>(p, d);
   D.x = psi;
   D.out = hpsi;
-  D.nq = 3;
+  D.nq = sums ? 3 : 0;
   return apply_op<T>(p->g, d, D, EPI_GRAD, p->acc, false, p->stream);
 }
 
 extern "C" gpe_status gpe_energy(gpe_plan p, const void* psi, double* E, double* mu, double* norm2) {
   if (!p || !psi) return fail(GPE_EINVAL, "plan or psi is NULL");
-  gpe_status s = p->prec == GPE_F32 ? do_grad<float>(p, *p->d32, psi, nullptr) : do_grad<double>(p, *p->d64, psi, nullptr);
+  gpe_status s = p->prec == GPE_F32 ? do_grad<float>(p, *p->d32, psi, nullptr, true)
+                                    : do_grad<double>(p, *p->d64, psi, nullptr, true);
   if (s != GPE_OK) return s;
   return read_energy(p, E, mu, norm2);
 }
@@ -345,7 +345,9 @@ extern "C" gpe_status gpe_energy(gpe_plan p, const void* psi, double* E, double*
 extern "C" gpe_status gpe_grad(gpe_plan p, const void* psi, void* hpsi, double* E, double* mu) {
   if (!p || !psi || !hpsi) return fail(GPE_EINVAL, "plan, psi or hpsi is NULL");
   if (psi == hpsi) return fail(GPE_EINVAL, "hpsi must not alias psi");
-  gpe_status s = p->prec == GPE_F32 ? do_grad<float>(p, *p->d32, psi, hpsi) : do_grad<double>(p, *p->d64, psi, hpsi);
+  const bool sums = E || mu;   // without them the reductions are left out
+  gpe_status s = p->prec == GPE_F32 ? do_grad<float>(p, *p->d32, psi, hpsi, sums)
+                                    : do_grad<double>(p, *p->d64, psi, hpsi, sums);
   if (s != GPE_OK) return s;
   if (E || mu) return read_energy(p, E, mu, nullptr);
   return GPE_OK;
@@ -372,9 +374,8 @@ extern "C" gpe_status gpe_hessvec(gpe_plan p, const void* psi, const void* dir, 
 
 template <typename T>
 static gpe_status do_step(gpe_plan p, const void* psi, const void* hpsi, double tau, void* out) {
-  gpe_status s = launch_moments<T>(psi, hpsi, p->g.M, p->g.nbatch, p->g.is_complex, p->sc, p->stream);
-  if (s != GPE_OK) return s;
-  s = launch_step_coef(p->sc.results, p->g.nbatch, p->g.hvol, tau, p->sc.coef, p->stream);
+  gpe_status s = launch_moments<T>(psi, hpsi, p->g.M, p->g.nbatch, p->g.is_complex, p->sc,
+                                   MomentCoef{1, p->g.hvol, tau, p->sc.coef}, p->stream);
   if (s != GPE_OK) return s;
   return launch_axpby<T>(psi, hpsi, p->sc.coef, 2, p->g.M, p->g.nbatch, out, p->g.is_complex, p->stream);
 }
@@ -394,9 +395,8 @@ template <typename T>
 static gpe_status do_prolong(gpe_plan c, gpe_plan f, const GridDev<T>& dc, const GridDev<T>& df, const void* in, void* out) {
   gpe_status s = launch_prolong<T>(c->g, f->g, dc, df, in, out, f->acc, f->tmp, f->stream);
   if (s != GPE_OK) return s;
-  s = launch_moments<T>(out, nullptr, f->g.M, f->g.nbatch, f->g.is_complex, f->sc, f->stream);
-  if (s != GPE_OK) return s;
-  s = launch_norm_coef(f->sc.results, f->g.nbatch, f->g.hvol, f->sc.coef, f->stream);
+  s = launch_moments<T>(out, nullptr, f->g.M, f->g.nbatch, f->g.is_complex, f->sc,
+                        MomentCoef{2, f->g.hvol, 0.0, f->sc.coef}, f->stream);
   if (s != GPE_OK) return s;
   return launch_axpby<T>(out, nullptr, f->sc.coef, 1, f->g.M, f->g.nbatch, out, f->g.is_complex, f->stream);
 }

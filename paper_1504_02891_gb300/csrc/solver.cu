@@ -16,7 +16,7 @@
 #include <memory>
 #include <type_traits>
 #include <vector>
-#include "gpe_internal.h"
+#include "ops_impl.cuh"
 
 namespace gpe {
 
@@ -384,9 +384,7 @@ static gpe_status alg1_run(Level<T>& L, int objective, int first_slot, int max_i
 // X in xs[slot] scaled to unit 2-norm.
 template <typename T>
 static gpe_status normalise_slot(Level<T>& L, int slot, cudaStream_t st) {
-  gpe_status s = launch_moments<T>(L.xs[slot], nullptr, L.M, 1, L.g.is_complex, L.sc, st);
-  if (s != GPE_OK) return s;
-  s = launch_norm_coef(L.sc.results, 1, 1.0, L.sc.coef, st);
+  gpe_status s = launch_moments<T>(L.xs[slot], nullptr, L.M, 1, L.g.is_complex, L.sc, MomentCoef{2, 1.0, 0.0, L.sc.coef}, st);
   if (s != GPE_OK) return s;
   return launch_axpby<T>(L.xs[slot], nullptr, L.sc.coef, 1, L.M, 1, L.xs[slot], L.g.is_complex, st);
 }
@@ -1287,9 +1285,7 @@ static gpe_status run_batch_group(BatchGroup& B, const std::vector<GridHost>& gh
     s = launch_convert<float, float>((const float*)psi[B.idx[k]], (float*)((char*)B.x + vbytes * k), nreal, sh, st);
     if (s != GPE_OK) return s;
   }
-  s = launch_moments<float>(B.x, nullptr, M, n, cplx, B.sc, st);
-  if (s != GPE_OK) return s;
-  s = launch_norm_coef(B.sc.results, n, 1.0, B.sc.coef, st);
+  s = launch_moments<float>(B.x, nullptr, M, n, cplx, B.sc, MomentCoef{2, 1.0, 0.0, B.sc.coef}, st);
   if (s != GPE_OK) return s;
   s = launch_axpby<float>(B.x, nullptr, B.sc.coef, 1, M, n, B.x, cplx, st);
   if (s != GPE_OK) return s;
