@@ -1183,6 +1183,9 @@ __global__ void __launch_bounds__(NTHREADS) k_alg1_persist(PersistArgs<T> P) {
 // ----------------------------------------------------------------- finite differences
 // H_lin of §2.1 per axis (3/5/7-point, zero Dirichlet values outside) with the
 // central-difference rotation term, then the same epilogue as the spectral pass.
+// Float64 is bound by the float64 pipe (2 operations a clock and SM): the
+// diagonal is one coefficient per point, V + sum 1/h^2, and each axis adds one
+// addition and one multiply-add.
 template <typename T, bool CPLX, int EPI>
 __global__ void __launch_bounds__(NTHREADS) k_fd(FDGeom G, const T* __restrict__ rx, const T* __restrict__ ry,
                                                 PassData<T> D) {
@@ -1201,34 +1204,54 @@ __global__ void __launch_bounds__(NTHREADS) k_fd(FDGeom G, const T* __restrict__
   for (int q = 0; q < NQ; ++q) acc_zero(acc[q]);
   T amax = T(0);
   const long long base = inst * G.M;
+  xin += base;
+  if (xsub) xsub += base;
   const T a0 = (T)G.ih2[0], a1 = (T)G.ih2[1], a2 = (T)G.ih2[2];
-  for (long long li = (long long)tb * blockDim.x + threadIdx.x; li < G.M; li += (long long)G.tiles * blockDim.x) {
-    const int i0 = (int)(li % G.n0);
-    const long long rest = li / G.n0;
-    const int i1 = (int)(rest % G.n1);
-    const int i2 = (int)(rest / G.n1);
-    auto ld = [&](long long k) -> V {
-      V v = xin[base + k];
-      if (xsub) v = v - xsub[base + k];
+  constexpr bool F64 = sizeof(T) == 8;
+  const T adiag = a0 + a1 + a2;                  // (axes beyond dim have ih2 = 0)
+  const T h0 = T(-0.5) * a0, h1 = T(-0.5) * a1, h2 = T(-0.5) * a2;
+  const unsigned int n0 = G.n0, n1 = G.n1, n2 = G.n2, s2 = n0 * n1, M = (unsigned int)G.M;
+  const unsigned int step = (unsigned int)G.tiles * blockDim.x;
+  for (unsigned int li = (unsigned int)tb * blockDim.x + threadIdx.x; li < M; li += step) {
+    const unsigned int row = li / n0, i0 = li - row * n0;
+    const unsigned int i2 = row / n1, i1 = row - i2 * n1;
+    auto ld = [&](unsigned int k) -> V {
+      V v = xin[k];
+      if (xsub) v = v - xsub[k];
       return v;
     };
     const V x = ld(li);
     V xm = i0 > 0 ? ld(li - 1) : vzero<V>();
-    V xp = i0 < G.n0 - 1 ? ld(li + 1) : vzero<V>();
-    V lin = (a0) * x - (T(0.5) * a0) * (xm + xp);
-    V dx = xp - xm;
-    V dy = vzero<V>();
-    if (G.dim >= 2) {
-      V ym = i1 > 0 ? ld(li - G.n0) : vzero<V>();
-      V yp = i1 < G.n1 - 1 ? ld(li + G.n0) : vzero<V>();
-      lin = lin + (a1) * x - (T(0.5) * a1) * (ym + yp);
-      dy = yp - ym;
-    }
-    if (G.dim >= 3) {
-      const long long s2 = (long long)G.n0 * G.n1;
-      V zm = i2 > 0 ? ld(li - s2) : vzero<V>();
-      V zp = i2 < G.n2 - 1 ? ld(li + s2) : vzero<V>();
-      lin = lin + (a2) * x - (T(0.5) * a2) * (zm + zp);
+    V xp = i0 < n0 - 1 ? ld(li + 1) : vzero<V>();
+    V dx = vzero<V>(), dy = vzero<V>(), lin;
+    if constexpr (F64) {
+      lin = (adiag + D.V[li]) * x + h0 * (xm + xp);
+      if constexpr (CPLX) dx = xp - xm;
+      if (G.dim >= 2) {
+        V ym = i1 > 0 ? ld(li - n0) : vzero<V>();
+        V yp = i1 < n1 - 1 ? ld(li + n0) : vzero<V>();
+        lin = lin + h1 * (ym + yp);
+        if constexpr (CPLX) dy = yp - ym;
+      }
+      if (G.dim >= 3) {
+        V zm = i2 > 0 ? ld(li - s2) : vzero<V>();
+        V zp = i2 < n2 - 1 ? ld(li + s2) : vzero<V>();
+        lin = lin + h2 * (zm + zp);
+      }
+    } else {
+      lin = (a0) * x - (T(0.5) * a0) * (xm + xp);
+      dx = xp - xm;
+      if (G.dim >= 2) {
+        V ym = i1 > 0 ? ld(li - n0) : vzero<V>();
+        V yp = i1 < n1 - 1 ? ld(li + n0) : vzero<V>();
+        lin = lin + (a1) * x - (T(0.5) * a1) * (ym + yp);
+        dy = yp - ym;
+      }
+      if (G.dim >= 3) {
+        V zm = i2 > 0 ? ld(li - s2) : vzero<V>();
+        V zp = i2 < n2 - 1 ? ld(li + s2) : vzero<V>();
+        lin = lin + (a2) * x - (T(0.5) * a2) * (zm + zp);
+      }
     }
     if constexpr (CPLX) {
       if (G.omega != 0.0) {
@@ -1242,8 +1265,8 @@ __global__ void __launch_bounds__(NTHREADS) k_fd(FDGeom G, const T* __restrict__
         lin = lin + iw;
       }
     }
-    lin = lin + D.V[li] * x;
-    epilogue_point<T, CPLX, EPI>(E, base + li, x, lin, acc, amax);
+    if constexpr (!F64) lin = lin + D.V[li] * x;
+    epilogue_point<T, CPLX, EPI, 2>(E, base + li, x, lin, acc, amax);
   }
   if (EPI == EPI_HESS || D.nq == 0) return;
   if (reduce_partials(acc, amax, D.nq, D.partials, D.results, D.ticket, G.tiles)) run_control<T>(D);
