@@ -244,10 +244,14 @@ struct LineFFT<double, LF> {
     }
   }
 
-  // T applied to the line (as LineFFT<float>::apply); ex.join(m, j) joins the
-  // line's magnitudes over its threads.
+  // A line in fixed point: its level (max < 2^m and L1 < 2^(m + l) in units of
+  // 2^(E - 1075 - (m - 53))) and whether it is finite.
+  struct Level {
+    int E, m, l;
+    bool finite;
+  };
   template <typename Ex>
-  __device__ __forceinline__ void apply(double2 (&v)[8], const Ex& ex, int& par, const LineSym<double, F>& sym) const {
+  __device__ __forceinline__ Level to_fixed(const double2 (&v)[8], I2 (&z)[8], const Ex& ex) const {
     LineMag mg;
     mg.E = 1;
 #pragma unroll
@@ -261,21 +265,37 @@ struct LineFFT<double, LF> {
 #pragma unroll
     for (int s = 0; s < 8; ++s) mg.S += top(v[s].x) + top(v[s].y);
     mg = ex.join(mg);
-    const bool finite = mg.E < 2047;
-    const int E = finite ? (int)mg.E : 1;
+    Level L;
+    L.finite = mg.E < 2047;
+    L.E = L.finite ? (int)mg.E : 1;
     const int b = 32 - __clz((int)mg.S);         // L1 < 2^(b + E - 1023 - 19)
-    // input level: max < 2^m, L1 < 2^(m + l).  A value is below 2^62 after one
-    // stage, after two, and in the spectrum
-    const int l = b - 20;
-    int m = min(61, min(62 - min(4, l), 62 + LOW - l));
-    if (N8 > 1) m = min(m, 64 - min(7, l));
-    const int base = m - 53;
-    I2 z[8];
+    // a value is below 2^62 after one stage, after two, and in the spectrum
+    L.l = b - 20;
+    L.m = min(61, min(62 - min(4, L.l), 62 + LOW - L.l));
+    if (N8 > 1) L.m = min(L.m, 64 - min(7, L.l));
 #pragma unroll
     for (int s = 0; s < 8; ++s) {
-      z[s].x = finite ? d2fix(v[s].x, E, base) : 0;
-      z[s].y = finite ? d2fix(v[s].y, E, base) : 0;
+      z[s].x = L.finite ? d2fix(v[s].x, L.E, L.m - 53) : 0;
+      z[s].y = L.finite ? d2fix(v[s].y, L.E, L.m - 53) : 0;
     }
+    return L;
+  }
+  // Back to double, conjugated; the value of one unit is 2^e.
+  static __device__ __forceinline__ void from_fixed(const I2 (&z)[8], double2 (&v)[8], int e, bool finite) {
+    const double bad = __longlong_as_double(0x7ff8000000000000LL);
+#pragma unroll
+    for (int s = 0; s < 8; ++s) {
+      v[s].x = finite ? fix2d(z[s].x, e) : bad;
+      v[s].y = finite ? -fix2d(z[s].y, e) : bad;
+    }
+  }
+
+  // T applied to the line (as LineFFT<float>::apply); ex.join(m) joins the
+  // line's magnitudes over its threads.
+  template <typename Ex>
+  __device__ __forceinline__ void apply(double2 (&v)[8], const Ex& ex, int& par, const LineSym<double, F>& sym) const {
+    I2 z[8];
+    const Level L = to_fixed(v, z, ex);
     // symbol (a p^2 + c p) 2^es with |a| + |c| <= 1, p in units of F/2
     const double pm = (double)(F / 2);
     const double a = sym.c2 * (sym.dl * pm) * (sym.dl * pm), c = sym.c1c * (sym.dl * pm);
@@ -284,7 +304,7 @@ struct LineFFT<double, LF> {
     // ||Y||_2^2 <= 2^R2 in the spectrum's units; mean square of the symbol
     // (a p^2 + c p over p in [-1, 1)): a^2/5 + c^2/3, and a little more on
     // short lines.  Later radix-8 stages grow by 1.5 bits and drop 2
-    const int R2 = LF + (m - LOW) + (m + l - LOW) + dexp(0.21 * a * a + 0.34 * c * c) - 1022 - 2 * es;
+    const int R2 = LF + (L.m - LOW) + (L.m + L.l - LOW) + dexp(0.21 * a * a + 0.34 * c * c) - 1022 - 2 * es;
     const int k = max(0, max((R2 + 4) >> 1, ((R2 + LF + 1) >> 1) - LOW) - 62);
     // a, c as fractions of 2^(62 - k): mantissas shifted from 2^(E - 1075)
     int ah, al, ch, cl;
@@ -310,14 +330,34 @@ struct LineFFT<double, LF> {
         }
       }
     }
-    // value of one unit: 2^(E - 1075 - base), the bits dropped, the symbol's 2^es
-    const int eo = E - 1075 - base + 2 * LOW + es + k;
-    const double bad = __longlong_as_double(0x7ff8000000000000LL);
+    // value of one unit: the line's, the bits dropped, the symbol's 2^es
+    from_fixed(z, v, L.E - 1075 - (L.m - 53) + 2 * LOW + es + k, L.finite);
+  }
+
+  // The line's midpoint values (prolong.cuh): forward transform, mode p times
+  // e^{i pi p / F}, inverse transform; fine: the table of 2F points.
+  template <typename Ex>
+  __device__ __forceinline__ void midpoints(double2 (&v)[8], const Ex& ex, int& par, const Tw* __restrict__ fine) const {
+    I2 z[8];
+    const Level L = to_fixed(v, z, ex);
+    const int R2 = LF + (L.m - LOW) + (L.m + L.l - LOW);   // unit symbol
+    const int k = max(0, max((R2 + 4) >> 1, ((R2 + LF + 1) >> 1) - LOW) - 62);
+    const long long h = (1LL << k) >> 1;
+#pragma unroll 1
+    for (int pass = 0; pass < 2; ++pass) {
+      forward(z, ex, par);
+      if (pass == 0) {
 #pragma unroll
-    for (int s = 0; s < 8; ++s) {
-      v[s].x = finite ? fix2d(z[s].x, eo) : bad;
-      v[s].y = finite ? -fix2d(z[s].y, eo) : bad;
+        for (int s = 0; s < 8; ++s) {
+          const int m = j + s * TPL;
+          const int p = m < (F >> 1) ? m : m - F;
+          const I2 c = fix_cmul<false>(mkI2(z[s].x, -z[s].y), __ldg(fine + (p & (2 * F - 1))));
+          const bool nyq = m == (F >> 1);
+          z[s] = mkI2(nyq ? 0 : (c.x + h) >> k, nyq ? 0 : (c.y + h) >> k);
+        }
+      }
     }
+    from_fixed(z, v, L.E - 1075 - (L.m - 53) + 2 * LOW + k - LF, L.finite);
   }
 };
 

@@ -121,7 +121,13 @@ template <typename T>
 gpe_status launch_inject(const GridHost& gf, const GridHost& gc, const void* f, void* c, cudaStream_t st);
 template <typename T>
 gpe_status launch_prolong(const GridHost& gc, const GridHost& gf, const GridDev<T>& dc, const GridDev<T>& df,
-                          const void* in, void* out, void* tmp1, void* tmp2, cudaStream_t st);
+                          const void* in, void* out, void* tmp1, void* tmp2, const double* coef, cudaStream_t st);
+// Cascadic transfer of unit-norm data: the axes, then the scale to unit norm
+// (h: cell volume of the fine grid's norm, sc: its scratch).
+template <typename T>
+gpe_status prolong_normalised(const GridHost& gc, const GridHost& gf, const GridDev<T>& dc, const GridDev<T>& df,
+                              const void* in, void* out, void* tmp1, void* tmp2, double h, Scratch& sc,
+                              cudaStream_t st);
 template <typename Ti, typename To>
 gpe_status launch_convert(const Ti* in, To* out, long long n, double scale, cudaStream_t st);
 gpe_status launch_to_shifted_f32(const double* xk, const double* gk, double th, float* xk32, float* pk32, long long n,

@@ -375,9 +375,18 @@ gpe_status launch_inject(const GridHost& gf, const GridHost& gc, const void* f, 
   return GPE_OK;
 }
 
+// Coarse axes whose lines the register kernels prolong (prolong.cuh); FD and
+// complex sine grids, and lines too short or too long, take the kernels below.
+static inline bool prolong_line_ok(const GridHost& gc, int a) { return line_axis_ok(gc, a) && gc.F[a] <= 512; }
+template <typename T>
+gpe_status launch_prolong_line(const GridHost& gc, int axis, const PassGeom<T>& G, const void* in, void* out,
+                               const double* coef, const GridDev<T>& df, cudaStream_t st);
+
+// `coef`: factor per instance that the last axis applies (null: none); only
+// where prolong_line_ok takes that axis.
 template <typename T>
 gpe_status launch_prolong(const GridHost& gc, const GridHost& gf, const GridDev<T>& dc, const GridDev<T>& df,
-                          const void* in, void* out, void* tmp1, void* tmp2, cudaStream_t st) {
+                          const void* in, void* out, void* tmp1, void* tmp2, const double* coef, cudaStream_t st) {
   int ext[3] = {gc.ext[0], gc.ext[1], gc.ext[2]};
   const void* src = in;
   for (int a = 0; a < gc.dim; ++a) {
@@ -387,7 +396,16 @@ gpe_status launch_prolong(const GridHost& gc, const GridHost& gf, const GridDev<
     const long long Mc = (long long)ext[0] * ext[1] * ext[2];
     const long long Mf = (long long)oext[0] * oext[1] * oext[2];
     ProfScope ps(kernel_name("prolong", sizeof(T) == 8, gc.is_complex, -1), st);
-    if (gc.disc == GPE_FD) {
+    const double* scale = a == gc.dim - 1 ? coef : nullptr;
+    if (prolong_line_ok(gc, a)) {
+      PassGeom<T> G = dc.geom[a];
+      G.n0 = ext[0];
+      G.n1 = ext[1];
+      G.n2 = ext[2];
+      G.M = Mc;
+      gpe_status s = launch_prolong_line<T>(gc, a, G, src, dst, scale, df, st);
+      if (s != GPE_OK) return s;
+    } else if (gc.disc == GPE_FD) {
       const long long n = Mf * gc.nbatch;
       if (gc.is_complex)
         k_prolong_fd_axis<T, true><<<ew_blocks(n), NTHREADS, 0, st>>>(src, dst, a, ext[0], ext[1], ext[2], gc.ext[a],
@@ -422,6 +440,28 @@ gpe_status launch_prolong(const GridHost& gc, const GridHost& gf, const GridDev<
     src = dst;
   }
   return GPE_OK;
+}
+
+// The transfer and its normalisation.  On sine grids the padded transform
+// keeps the discrete norm (Parseval, no Nyquist mode), so the scale comes from
+// the coarse data, 1/2^dim of the fine, and the last axis applies it; on other
+// grids it takes two more passes over the fine data.
+template <typename T>
+gpe_status prolong_normalised(const GridHost& gc, const GridHost& gf, const GridDev<T>& dc, const GridDev<T>& df,
+                              const void* in, void* out, void* tmp1, void* tmp2, double h, Scratch& sc,
+                              cudaStream_t st) {
+  const bool early = gc.disc == GPE_SINE && prolong_line_ok(gc, gc.dim - 1);
+  if (early) {
+    const double hc = h * (double)(1 << gc.dim);
+    gpe_status s = launch_moments<T>(in, nullptr, gc.M, gc.nbatch, gc.is_complex, sc, MomentCoef{2, hc, 0.0, sc.coef}, st);
+    if (s != GPE_OK) return s;
+    return launch_prolong<T>(gc, gf, dc, df, in, out, tmp1, tmp2, sc.coef, st);
+  }
+  gpe_status s = launch_prolong<T>(gc, gf, dc, df, in, out, tmp1, tmp2, nullptr, st);
+  if (s != GPE_OK) return s;
+  s = launch_moments<T>(out, nullptr, gf.M, gf.nbatch, gf.is_complex, sc, MomentCoef{2, h, 0.0, sc.coef}, st);
+  if (s != GPE_OK) return s;
+  return launch_axpby<T>(out, nullptr, sc.coef, 1, gf.M, gf.nbatch, out, gf.is_complex, st);
 }
 
 // 2D Fourier grids: the register-FFT line kernels (lines2d.cuh); *handled is
@@ -596,7 +636,9 @@ gpe_status launch_alg1_persist(const GridHost& g, const GridDev<T>& d, const Pas
                                       cudaStream_t);                                                               \
   template gpe_status launch_inject<T>(const GridHost&, const GridHost&, const void*, void*, cudaStream_t);         \
   template gpe_status launch_prolong<T>(const GridHost&, const GridHost&, const GridDev<T>&, const GridDev<T>&,     \
-                                        const void*, void*, void*, void*, cudaStream_t);                           \
+                                        const void*, void*, void*, void*, const double*, cudaStream_t);            \
+  template gpe_status prolong_normalised<T>(const GridHost&, const GridHost&, const GridDev<T>&, const GridDev<T>&, \
+                                            const void*, void*, void*, void*, double, Scratch&, cudaStream_t);     \
   template gpe_status apply_op<T>(const GridHost&, const GridDev<T>&, PassData<T>, int, void*, bool, cudaStream_t); \
   template gpe_status persist_config<T>(const GridHost&, const GridDev<T>&, int, int*, size_t*);                      \
   template gpe_status launch_alg1_persist<T>(const GridHost&, const GridDev<T>&, const PassData<T>&, void*,         \

@@ -393,12 +393,7 @@ extern "C" gpe_status gpe_feasible_step(gpe_plan p, const void* psi, const void*
 
 template <typename T>
 static gpe_status do_prolong(gpe_plan c, gpe_plan f, const GridDev<T>& dc, const GridDev<T>& df, const void* in, void* out) {
-  gpe_status s = launch_prolong<T>(c->g, f->g, dc, df, in, out, f->acc, f->tmp, f->stream);
-  if (s != GPE_OK) return s;
-  s = launch_moments<T>(out, nullptr, f->g.M, f->g.nbatch, f->g.is_complex, f->sc,
-                        MomentCoef{2, f->g.hvol, 0.0, f->sc.coef}, f->stream);
-  if (s != GPE_OK) return s;
-  return launch_axpby<T>(out, nullptr, f->sc.coef, 1, f->g.M, f->g.nbatch, out, f->g.is_complex, f->stream);
+  return prolong_normalised<T>(c->g, f->g, dc, df, in, out, f->acc, f->tmp, f->g.hvol, f->sc, f->stream);
 }
 
 extern "C" gpe_status gpe_prolong(gpe_plan c, gpe_plan f, const void* psi_c, void* psi_f) {

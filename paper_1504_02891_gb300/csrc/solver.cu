@@ -829,9 +829,7 @@ static gpe_status load_initial(gpe_plan plan, SolverCache& C, Level<T>& L0, cons
 
 template <typename T>
 static gpe_status prolong_into(Level<T>& Lc, Level<T>& Lf, cudaStream_t st) {
-  gpe_status s = launch_prolong<T>(Lc.g, Lf.g, Lc.d, Lf.d, Lc.xk, Lf.xs[0], Lf.acc, Lf.gs[0], st);
-  if (s != GPE_OK) return s;
-  return normalise_slot0<T>(Lf, st);
+  return prolong_normalised<T>(Lc.g, Lf.g, Lc.d, Lf.d, Lc.xk, Lf.xs[0], Lf.acc, Lf.gs[0], 1.0, Lf.sc, st);
 }
 
 template <typename T>
