@@ -31,6 +31,9 @@
 // hardware barriers; every CTA executes the same sequence of them because the
 // control decisions are bit-identical across the cluster.
 #include <cooperative_groups.h>
+#include <map>
+#include <mutex>
+#include <tuple>
 #include "ops_impl.cuh"
 #include "linefft.cuh"
 
@@ -663,6 +666,28 @@ static int ilog2i(int v) {
   return l;
 }
 
+// The attributes of one cluster shape of a kernel and how many such clusters
+// the device holds, set and looked up once per device and shape (three host
+// calls on every launch otherwise).
+static cudaError_t cluster_limits(const void* fn, int cs, size_t smem, const cudaLaunchConfig_t& cfg, int* maxc) {
+  static std::mutex mu;
+  static std::map<std::tuple<int, const void*, int, size_t>, int> known;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  std::lock_guard<std::mutex> lk(mu);
+  const auto key = std::make_tuple(dev, fn, cs, smem);
+  const auto it = known.find(key);
+  if (it != known.end()) {
+    *maxc = it->second;
+    return cudaSuccess;
+  }
+  cudaError_t e = raise_smem(fn, smem);
+  if (e == cudaSuccess && cs > 8) e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(maxc, fn, &cfg);
+  if (e == cudaSuccess) known[key] = *maxc;
+  return e;
+}
+
 // Launch the cluster engine for `ninst` instances of one grid; clusters loop
 // over instances.  Returns GPE_EINVAL if the grid does not fit (callers then
 // use the CTA-grid path).
@@ -685,8 +710,6 @@ gpe_status launch_cluster_alg1(ClusterArgs A, int cplx, cudaStream_t st) {
   A.vpot_bytes = vp;
   const void* fn = A.shifted ? (cplx ? cluster_fn<true, true>(lf) : cluster_fn<false, true>(lf))
                              : (cplx ? cluster_fn<true, false>(lf) : cluster_fn<false, false>(lf));
-  GPE_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  if (cs > 8) GPE_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -698,9 +721,9 @@ gpe_status launch_cluster_alg1(ClusterArgs A, int cplx, cudaStream_t st) {
   cfg.stream = st;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  int maxc = 0;
   cfg.gridDim = dim3(cs);
-  GPE_CUDA(cudaOccupancyMaxActiveClusters(&maxc, fn, &cfg));
+  int maxc = 0;
+  GPE_CUDA(cluster_limits(fn, cs, smem, cfg, &maxc));
   if (maxc < 1) return fail(GPE_EINVAL, "no cluster of this shape fits on the device");
   const int ncl = std::min(A.ninst, maxc);
   cfg.gridDim = dim3(cs * ncl);

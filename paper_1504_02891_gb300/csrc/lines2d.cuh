@@ -328,17 +328,6 @@ __global__ void __launch_bounds__(lines_x_threads<T>(LF), lines_x_minb<T>(LF)) k
   if (reduce_partials(acc, amax, D.nq, D.partials, D.results, D.ticket, tiles_per_inst)) run_control<T>(D);
 }
 
-static int num_sms() {
-  static int n = 0;
-  if (n == 0) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    if (n <= 0) n = 152;
-  }
-  return n;
-}
-
 template <typename T, bool CPLX, int EPI, int LF0>
 static gpe_status launch_lines_x(const GridDev<T>& d, const PassData<T>& Dx, int nbatch, int groups,
                                  cudaStream_t st) {
@@ -350,16 +339,11 @@ static gpe_status launch_lines_x(const GridDev<T>& d, const PassData<T>& Dx, int
   const size_t vsz = sizeof(T) * (CPLX ? 2 : 1);
   const size_t smem = ((size_t)(1 << LF0) + 2 * (size_t)NL * LineFFT<T, LF0>::P) * sizeof(C) +
                       3 * (size_t)NV * NTX * vsz + (size_t)NV * NTX * sizeof(T);
-  static int occ = -1;
-  if (occ < 0) {
-    GPE_CUDA(cudaFuncSetAttribute(k_lines_x<T, CPLX, EPI, LF0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)smem));
-    GPE_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_lines_x<T, CPLX, EPI, LF0>, NTX, smem));
-    if (occ < 1) occ = 1;
-  }
+  static const KernelShape sh = kernel_shape((const void*)k_lines_x<T, CPLX, EPI, LF0>, NTX, smem);
+  GPE_CUDA(sh.e);
   // a few resident waves in all (4, or the measured choice), at most the
   // reduction scratch's capacity
-  const long long want = (long long)tuned_waves(0, sizeof(T) == 8, CPLX, gx.n0, gx.n1, nbatch) * occ * num_sms();
+  const long long want = (long long)tuned_waves(0, sizeof(T) == 8, CPLX, gx.n0, gx.n1, nbatch) * sh.occ * num_sms();
   int tiles = groups;
   while (tiles > 1 && (long long)tiles * nbatch > want) tiles = (tiles + 1) / 2;
   while (tiles > 1 && (long long)tiles * nbatch > d.max_blocks) tiles = (tiles + 1) / 2;
@@ -392,14 +376,10 @@ static gpe_status launch_lines2d_t(const GridDev<T>& d, const PassData<T>& D, in
     Dy.nq = 0;
     Dy.control = 0;
     const size_t smem = ((size_t)(1 << LF1) * (1 + 2 * CW) + 16 * (size_t)YT) * sizeof(C);
-    static int occ = -1;
-    if (occ < 0) {
-      GPE_CUDA(cudaFuncSetAttribute(k_lines_y<T, CPLX, LF1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      GPE_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_lines_y<T, CPLX, LF1>, YT, smem));
-      if (occ < 1) occ = 1;
-    }
+    static const KernelShape sh = kernel_shape((const void*)k_lines_y<T, CPLX, LF1>, YT, smem);
+    GPE_CUDA(sh.e);
     const int total = nbatch * colgroups;
-    const int grid = std::min(total, tuned_waves(1, sizeof(T) == 8, CPLX, gx.n0, gx.n1, nbatch) * occ * num_sms());
+    const int grid = std::min(total, tuned_waves(1, sizeof(T) == 8, CPLX, gx.n0, gx.n1, nbatch) * sh.occ * num_sms());
     ProfScope ps(kernel_name("linesy", sizeof(T) == 8, CPLX, EPI_ACC, gx.M * nbatch), st);
     k_lines_y<T, CPLX, LF1><<<grid, YT, smem, st>>>(gy, Dy, colgroups, total);
     GPE_CUDA(cudaGetLastError());

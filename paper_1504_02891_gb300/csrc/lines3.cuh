@@ -332,7 +332,7 @@ static gpe_status launch_axis_s_t(const GridDev<T>& d, int axis, const PassData<
   const PassGeom<T>& G = d.geom[axis];
   constexpr int CW = axs_cw<T>(LF), NT = axs_threads<T>(LF);
   const size_t smem = (size_t)FFT::F * sizeof(typename FFT::Tw) + 2 * (size_t)FFT::F * CW * sizeof(typename FFT::X);
-  static const cudaError_t allowed = allow_smem(k_axis_s<T, KIND, LF>, smem);
+  static const cudaError_t allowed = raise_smem((const void*)k_axis_s<T, KIND, LF>, smem);
   GPE_CUDA(allowed);
   const int width = axis == 1 ? G.n0 : G.n0 * G.n1;
   const int planes = nbatch * (axis == 1 ? G.n2 : 1);
@@ -353,17 +353,7 @@ static gpe_status launch_axis_x_t(const GridDev<T>& d, const PassData<T>& D, int
   const size_t vsz = sizeof(T) * (KIND == LK_CPLX ? 2 : 1);
   const size_t smem = (size_t)FFT::F * sizeof(typename FFT::Tw) + 2 * (size_t)NL * FFT::P * sizeof(typename FFT::X) +
                       (sizeof(T) == 8 ? (size_t)NV * NT * (2 * vsz + sizeof(T)) : 0);
-  struct Shape {
-    cudaError_t e;
-    int occ;
-  };
-  static const Shape sh = [&] {
-    Shape r{allow_smem(k_axis_x<T, KIND, EPI, LF>, smem), 1};
-    if (r.e == cudaSuccess)
-      r.e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r.occ, k_axis_x<T, KIND, EPI, LF>, NT, smem);
-    if (r.occ < 1) r.occ = 1;
-    return r;
-  }();
+  static const KernelShape sh = kernel_shape((const void*)k_axis_x<T, KIND, EPI, LF>, NT, smem);
   GPE_CUDA(sh.e);
   const long long rows = G.M / G.len;
   const long long lines = KIND == LK_CPLX ? rows : (rows + 1) / 2;

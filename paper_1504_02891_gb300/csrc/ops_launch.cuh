@@ -249,13 +249,6 @@ void GridDev<T>::destroy() {
   fsync = nullptr;
 }
 
-// Opt in to `bytes` of dynamic shared memory (static shared memory counts
-// against the 48 KiB default too, so the opt-in is requested for any size).
-template <typename K>
-static cudaError_t allow_smem(K kernel, size_t bytes) {
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 template <typename T, bool CPLX, int EPI>
 static gpe_status launch_pass_t(const PassGeom<T>& G, int blocks, const PassData<T>& D, cudaStream_t st) {
   using C = typename C2t<T>::type;
@@ -263,11 +256,7 @@ static gpe_status launch_pass_t(const PassGeom<T>& G, int blocks, const PassData
   const int nst = 1 + ((D.xsub || D.step_on_load) ? 1 : 0) + (D.acc_in ? 1 : 0);
   const size_t smem = (size_t)G.F * sizeof(C) + 2 * (size_t)G.LC * G.P * sizeof(C) +
                       (size_t)nst * G.LB * G.len * vsz + (EPI != EPI_ACC ? (size_t)G.LB * G.len * sizeof(T) : 0);
-  static size_t allowed = 0;
-  if (smem > allowed) {
-    GPE_CUDA(allow_smem(k_pass<T, CPLX, EPI>, smem));
-    allowed = smem;
-  }
+  GPE_CUDA(raise_smem((const void*)k_pass<T, CPLX, EPI>, smem));
   ProfScope ps(kernel_name("pass", sizeof(T) == 8, CPLX, EPI, G.M * (blocks / G.tiles)), st);
   k_pass<T, CPLX, EPI><<<blocks, G.nthreads, smem, st>>>(G, D);
   GPE_CUDA(cudaGetLastError());
@@ -424,13 +413,11 @@ gpe_status launch_prolong(const GridHost& gc, const GridHost& gf, const GridDev<
       const long long ostride_f = a == 1 ? (long long)oext[0] * oext[1] : (long long)oext[0];
       const int Ff = gf.F[a];
       if (gc.is_complex) {
-        static size_t allowed_c = 0;
-        if (smem > allowed_c) { GPE_CUDA(allow_smem(k_prolong_axis<T, true>, smem)); allowed_c = smem; }
+        GPE_CUDA(raise_smem((const void*)k_prolong_axis<T, true>, smem));
         k_prolong_axis<T, true><<<blocks, NTHREADS, smem, st>>>(G, Ff, ilog2(Ff), df.tw[a], gf.ext[a], stride_f,
                                                                 ostride_f, Mf, src, dst);
       } else {
-        static size_t allowed_r = 0;
-        if (smem > allowed_r) { GPE_CUDA(allow_smem(k_prolong_axis<T, false>, smem)); allowed_r = smem; }
+        GPE_CUDA(raise_smem((const void*)k_prolong_axis<T, false>, smem));
         k_prolong_axis<T, false><<<blocks, NTHREADS, smem, st>>>(G, Ff, ilog2(Ff), df.tw[a], gf.ext[a], stride_f,
                                                                  ostride_f, Mf, src, dst);
       }
@@ -585,7 +572,7 @@ gpe_status persist_config(const GridHost& g, const GridDev<T>& d, int epi, int* 
   const void* fn = nullptr;
   if (epi == EPI_F) fn = g.is_complex ? (const void*)k_alg1_persist<T, true, EPI_F> : (const void*)k_alg1_persist<T, false, EPI_F>;
   else fn = g.is_complex ? (const void*)k_alg1_persist<T, true, EPI_W> : (const void*)k_alg1_persist<T, false, EPI_W>;
-  GPE_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  GPE_CUDA(raise_smem(fn, smem));
   GPE_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, NTHREADS, smem));
   if (occ < 1) return GPE_OK;
   *grid = std::min(maxb, occ * nsm);

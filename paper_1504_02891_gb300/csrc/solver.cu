@@ -12,8 +12,15 @@
 #include <stdio.h>
 #include <stdlib.h>
 #include <string.h>
+#include <algorithm>
 #include <chrono>
+#include <map>
 #include <memory>
+#include <mutex>
+#include <new>
+#include <string>
+#include <system_error>
+#include <thread>
 #include <type_traits>
 #include <vector>
 #include "ops_impl.cuh"
@@ -27,6 +34,9 @@ struct Level {
   Scratch sc;
   long long M = 0;
   size_t bytes = 0;
+  void* vectors = nullptr;   // the allocations behind the pointers below
+  void* blocks = nullptr;
+  void* pinned = nullptr;
   void* acc = nullptr;
   void* xs[3] = {nullptr, nullptr, nullptr};
   void* gs[3] = {nullptr, nullptr, nullptr};
@@ -58,29 +68,48 @@ struct Level {
     if (s != GPE_OK) return s;
     s = sc.create(d.max_blocks, 1);
     if (s != GPE_OK) return s;
-    GPE_CUDA(cudaMalloc(&acc, bytes));
+    // one allocation for the nine vectors, one for the small device blocks, one
+    // pinned: a batch makes a pair of levels for every refinement in flight
+    const size_t vb = (bytes + 255) & ~(size_t)255;
+    GPE_CUDA(cudaMalloc(&vectors, 9 * vb));
+    char* v = static_cast<char*>(vectors);
+    acc = v;
     for (int i = 0; i < 3; ++i) {
-      GPE_CUDA(cudaMalloc(&xs[i], bytes));
-      GPE_CUDA(cudaMalloc(&gs[i], bytes));
+      xs[i] = v + (1 + i) * vb;
+      gs[i] = v + (4 + i) * vb;
     }
-    GPE_CUDA(cudaMalloc(&xk, bytes));
-    GPE_CUDA(cudaMalloc(&gk, bytes));
-    GPE_CUDA(cudaMalloc(&d_xs, sizeof(void*) * 3));
-    GPE_CUDA(cudaMalloc(&d_gs, sizeof(void*) * 3));
-    GPE_CUDA(cudaMemcpy(d_xs, xs, sizeof(void*) * 3, cudaMemcpyHostToDevice));
-    GPE_CUDA(cudaMemcpy(d_gs, gs, sizeof(void*) * 3, cudaMemcpyHostToDevice));
-    GPE_CUDA(cudaMalloc(&ctl, sizeof(Alg1Ctl)));
-    GPE_CUDA(cudaMalloc(&rn, sizeof(RNCtl)));
-    GPE_CUDA(cudaMalloc(&bar, 2 * sizeof(unsigned int)));
-    {
-      const float om = (float)g.omega;
-      GPE_CUDA(cudaMalloc(&d_omega, sizeof(float)));
-      GPE_CUDA(cudaMemcpy(d_omega, &om, sizeof(float), cudaMemcpyHostToDevice));
+    xk = v + 7 * vb;
+    gk = v + 8 * vb;
+    constexpr size_t CB = (sizeof(Alg1Ctl) + 255) & ~(size_t)255, RB = (sizeof(RNCtl) + 255) & ~(size_t)255;
+    GPE_CUDA(cudaMalloc(&blocks, CB + RB + 256));
+    char* q = static_cast<char*>(blocks);
+    ctl = reinterpret_cast<Alg1Ctl*>(q);
+    rn = reinterpret_cast<RNCtl*>(q + CB);
+    struct Small {
+      void* xs[3];
+      void* gs[3];
+      unsigned int bar[2];
+      int err;
+      float omega;
+    } sm = {};
+    static_assert(sizeof(Small) <= 256, "small block");
+    for (int i = 0; i < 3; ++i) {
+      sm.xs[i] = xs[i];
+      sm.gs[i] = gs[i];
     }
-    GPE_CUDA(cudaMalloc(&err, sizeof(int)));
-    GPE_CUDA(cudaMallocHost(&h_err, sizeof(int)));
-    GPE_CUDA(cudaMallocHost(&h_ctl, sizeof(Alg1Ctl)));
-    GPE_CUDA(cudaMallocHost(&h_rn, sizeof(RNCtl)));
+    sm.omega = (float)g.omega;
+    Small* ds = reinterpret_cast<Small*>(q + CB + RB);
+    GPE_CUDA(cudaMemcpy(ds, &sm, sizeof(sm), cudaMemcpyHostToDevice));
+    d_xs = ds->xs;
+    d_gs = ds->gs;
+    bar = ds->bar;
+    err = &ds->err;
+    d_omega = &ds->omega;
+    GPE_CUDA(cudaMallocHost(&pinned, CB + RB + 64));
+    char* h = static_cast<char*>(pinned);
+    h_ctl = reinterpret_cast<Alg1Ctl*>(h);
+    h_rn = reinterpret_cast<RNCtl*>(h + CB);
+    h_err = reinterpret_cast<int*>(h + CB + RB);
     memset(h_ctl, 0, sizeof(Alg1Ctl));
     memset(h_rn, 0, sizeof(RNCtl));
     return GPE_OK;
@@ -90,23 +119,10 @@ struct Level {
       if (chunk_exec[i]) cudaGraphExecDestroy(chunk_exec[i]);
     d.destroy();
     sc.destroy();
-    cudaFree(acc);
-    for (int i = 0; i < 3; ++i) {
-      cudaFree(xs[i]);
-      cudaFree(gs[i]);
-    }
-    cudaFree(xk);
-    cudaFree(gk);
-    cudaFree(d_xs);
-    cudaFree(d_gs);
-    cudaFree(ctl);
-    cudaFree(rn);
-    cudaFree(bar);
-    cudaFree(err);
-    cudaFree(d_omega);
-    cudaFreeHost(h_err);
-    cudaFreeHost(h_ctl);
-    cudaFreeHost(h_rn);
+    cudaFree(vectors);
+    cudaFree(blocks);
+    cudaFreeHost(pinned);
+    vectors = blocks = pinned = nullptr;
   }
   PassData<T> solver_data(int objective) const {
     PassData<T> D{};
@@ -1195,7 +1211,14 @@ struct BatchGroup {
   float* omega = nullptr;
   Alg1Ctl* ctl = nullptr;
   unsigned int* next = nullptr;
+  std::vector<Alg1Ctl> hc;      // the instances' control blocks
+  cudaStream_t st = nullptr;    // the groups' float32 stages run side by side
+  std::chrono::steady_clock::time_point t0;
   ~BatchGroup() {
+    if (st) {
+      cudaStreamSynchronize(st);
+      cudaStreamDestroy(st);
+    }
     d.destroy();
     sc.destroy();
     cudaFree(x);
@@ -1211,12 +1234,13 @@ struct BatchGroup {
 // same grid (extents, box, complexity): its potential, beta and Omega.  The
 // level's cached CUDA graphs captured the old operator and are dropped.
 template <typename T>
-static gpe_status level_set_problem(Level<T>& L, const GridHost& gi) {
+static gpe_status level_set_problem(Level<T>& L, const GridHost& gi, cudaStream_t st) {
   L.g.beta = gi.beta;
   L.g.omega = gi.omega;
   std::vector<T> hv((size_t)L.M);
   for (long long i = 0; i < L.M; ++i) hv[(size_t)i] = (T)gi.V[(size_t)i];
-  GPE_CUDA(cudaMemcpy(L.d.V, hv.data(), sizeof(T) * hv.size(), cudaMemcpyHostToDevice));
+  // (pageable: returns once the values are staged; ordered on the lane's stream)
+  GPE_CUDA(cudaMemcpyAsync(L.d.V, hv.data(), sizeof(T) * hv.size(), cudaMemcpyHostToDevice, st));
   if (L.g.disc != GPE_FD) {
     for (int a = 0; a < 2 && a < L.g.dim; ++a) {
       PassGeom<T>& G = L.d.geom[a];
@@ -1231,7 +1255,7 @@ static gpe_status level_set_problem(Level<T>& L, const GridHost& gi) {
   }
   L.d.fd.omega = gi.omega;
   const float om = (float)gi.omega;
-  GPE_CUDA(cudaMemcpy(L.d_omega, &om, sizeof(float), cudaMemcpyHostToDevice));
+  GPE_CUDA(cudaMemcpyAsync(L.d_omega, &om, sizeof(float), cudaMemcpyHostToDevice, st));
   for (int i = 0; i < 3; ++i)
     if (L.chunk_exec[i]) {
       cudaGraphExecDestroy(L.chunk_exec[i]);
@@ -1245,8 +1269,12 @@ static bool same_grid(const GridHost& a, const GridHost& b) {
          a.lo[1] == b.lo[1] && a.hi[0] == b.hi[0] && a.hi[1] == b.hi[1];
 }
 
-static gpe_status run_batch_group(BatchGroup& B, const std::vector<GridHost>& gh, void* const* psi,
-                                  const SolveParams& P, gpe_solve_report* reports, cudaStream_t st) {
+// The float32 stage of one group, queued on the group's own stream: the
+// instances' potentials and controls, their unit-norm data, one cluster launch,
+// the states back to psi and the control blocks to the host.
+static gpe_status queue_batch_group(BatchGroup& B, const std::vector<GridHost>& gh, void* const* psi,
+                                    const SolveParams& P) {
+  const cudaStream_t st = B.st;
   const int n = (int)B.idx.size();
   const GridHost& g = B.g;
   const long long M = g.M;
@@ -1266,7 +1294,8 @@ static gpe_status run_batch_group(BatchGroup& B, const std::vector<GridHost>& gh
   GPE_CUDA(cudaMalloc(&B.next, sizeof(unsigned int)));
   // per-instance potential, Omega and control (alpha = beta / (2 h_vol))
   std::vector<float> hv((size_t)M * n), hom(n);
-  std::vector<Alg1Ctl> hc(n);
+  std::vector<Alg1Ctl>& hc = B.hc;
+  hc.resize(n);
   for (int k = 0; k < n; ++k) {
     const GridHost& gi = gh[B.idx[k]];
     for (long long i = 0; i < M; ++i) hv[(size_t)k * M + i] = (float)gi.V[i];
@@ -1307,18 +1336,25 @@ static gpe_status run_batch_group(BatchGroup& B, const std::vector<GridHost>& gh
   A.ctl = B.ctl;
   A.results = B.sc.results;
   A.next = B.next;
-  auto t0 = std::chrono::steady_clock::now();
+  B.t0 = std::chrono::steady_clock::now();
   s = launch_cluster_alg1(A, cplx, st);
   if (s != GPE_OK) return s;
-  // results back to psi (physical units) and the reports
+  // results back to psi (physical units)
   for (int k = 0; k < n; ++k) {
     s = launch_convert<float, float>((const float*)((char*)B.x + vbytes * k), (float*)psi[B.idx[k]], nreal, 1.0 / sh,
                                      st);
     if (s != GPE_OK) return s;
   }
-  GPE_CUDA(cudaMemcpyAsync(hc.data(), B.ctl, sizeof(Alg1Ctl) * n, cudaMemcpyDeviceToHost, st));
-  GPE_CUDA(cudaStreamSynchronize(st));
-  const double ms32 = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count() / n;
+  return GPE_OK;
+}
+
+// Wait for the group's float32 stage and fill its reports.
+static gpe_status finish_batch_group(BatchGroup& B, const SolveParams& P, gpe_solve_report* reports) {
+  const int n = (int)B.idx.size();
+  std::vector<Alg1Ctl>& hc = B.hc;
+  GPE_CUDA(cudaMemcpyAsync(hc.data(), B.ctl, sizeof(Alg1Ctl) * n, cudaMemcpyDeviceToHost, B.st));
+  GPE_CUDA(cudaStreamSynchronize(B.st));
+  const double ms32 = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - B.t0).count() / n;
   for (int k = 0; k < n; ++k) {
     const Alg1Ctl& c = hc[k];
     gpe_solve_report& r = reports[B.idx[k]];
@@ -1333,73 +1369,171 @@ static gpe_status run_batch_group(BatchGroup& B, const std::vector<GridHost>& gh
     r.nfe = c.nfe;
     r.ms_f32 = ms32;
   }
-  if (!P.refine) return GPE_OK;
-  // float64 refinement (the mixed schedule's finest level, per instance):
-  // Algorithm 2 with float64 outer quantities and float32 difference-form
-  // subproblems in the cluster engine, from the float32 state, for every
-  // instance that did not reach res_tol
-  struct LevelPair {
-    Level<double> d;
-    Level<float> f;
-    ~LevelPair() {
-      d.destroy();
-      f.destroy();
-    }
-  };
-  std::unique_ptr<LevelPair> LP(new LevelPair());
-  Level<double>* Ld = &LP->d;
-  Level<float>* Lf = &LP->f;
-  s = Ld->create(g);
-  if (s == GPE_OK) s = Lf->create(g);
-  if (s != GPE_OK) return s;
-  // the refinement captures CUDA graphs, which the caller's stream may not
-  // allow (the legacy default stream cannot be captured): it runs on a
-  // private stream, after the work queued so far and before anything queued
-  // on the caller's stream later
-  struct PrivStream {
-    cudaStream_t s = nullptr;
-    cudaEvent_t e = nullptr;
-    ~PrivStream() {
-      if (e) cudaEventDestroy(e);
-      if (s) cudaStreamDestroy(s);
-    }
-  } ps;
-  GPE_CUDA(cudaStreamCreateWithFlags(&ps.s, cudaStreamNonBlocking));
-  GPE_CUDA(cudaEventCreateWithFlags(&ps.e, cudaEventDisableTiming));
-  GPE_CUDA(cudaEventRecord(ps.e, st));
-  GPE_CUDA(cudaStreamWaitEvent(ps.s, ps.e, 0));
-  const cudaStream_t caller = st;
-  st = ps.s;
-  for (int k = 0; k < n; ++k) {
-    gpe_solve_report& r = reports[B.idx[k]];
-    if (r.status == GPE_ENONFINITE || r.status == GPE_OK) continue;
-    const GridHost& gi = gh[B.idx[k]];
-    auto t1 = std::chrono::steady_clock::now();
-    s = level_set_problem<double>(*Ld, gi);
-    if (s == GPE_OK) s = level_set_problem<float>(*Lf, gi);
-    if (s != GPE_OK) return s;
-    s = launch_convert<float, double>((const float*)((char*)B.x + vbytes * k), (double*)Ld->xs[0], nreal, 1.0, st);
-    if (s == GPE_OK) s = normalise_slot0<double>(*Ld, st);
-    if (s != GPE_OK) return s;
-    LevelStats l2;
-    s = rn_run<double>(*Ld, P, 0, false, st, l2, 2.0 * r.mu, Lf);
-    if (s != GPE_OK) return s;
-    s = launch_convert<double, float>((const double*)Ld->xk, (float*)psi[B.idx[k]], nreal, 1.0 / sh, st);
-    if (s != GPE_OK) return s;
-    GPE_CUDA(cudaStreamSynchronize(st));
-    r.E = l2.F;
-    r.mu = 0.5 * l2.theta;
-    r.res = 0.5 * l2.res;
-    r.status = l2.converged ? GPE_OK : GPE_ENOCONV;
-    r.outer_f64 = l2.outer;
-    r.inner_f64 = l2.inner;
-    r.inner_f32 += l2.inner32;
-    r.nfe += l2.nfe;
-    r.ms_f64 = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t1).count();
+  return GPE_OK;
+}
+
+// Float64 refinement of instances (the mixed schedule's finest level, per
+// instance): Algorithm 2 with float64 outer quantities and float32
+// difference-form subproblems in the cluster engine, from the float32 state.
+//
+// An instance is a chain of small launches, each on at most one cluster (16 of
+// the 152 SMs), with a host decision after every outer step, so instances run
+// side by side: up to REFINE_LANES host threads, each with its own stream,
+// taking the next instance from a common list (largest grids first).  A lane
+// keeps a level pair of a grid for its next instance of that grid in the
+// pool; the pool holds at most one pair per lane and grid and ends with the
+// call.  24 instances 64^2..256^2: 239 ms one after another.
+constexpr int REFINE_LANES = 8;   // clusters of 16 CTAs that the device's GPCs hold
+
+struct LevelPair {
+  Level<double> d;
+  Level<float> f;
+  ~LevelPair() {
+    d.destroy();
+    f.destroy();
   }
-  GPE_CUDA(cudaEventRecord(ps.e, st));
-  GPE_CUDA(cudaStreamWaitEvent(caller, ps.e, 0));
+};
+
+struct RefinePool {
+  std::mutex mu;
+  std::vector<std::pair<BatchGroup*, int>> todo;   // (group, instance within it)
+  size_t next = 0;
+  std::map<BatchGroup*, std::vector<std::unique_ptr<LevelPair>>> idle;
+  gpe_status status = GPE_OK;
+  std::string error;
+  int device = 0;
+};
+
+static gpe_status refine_instance(BatchGroup& B, int k, LevelPair& LP, const std::vector<GridHost>& gh,
+                                  void* const* psi, const SolveParams& P, gpe_solve_report& r, cudaStream_t st) {
+  const GridHost& gi = gh[B.idx[k]];
+  const long long nreal = B.g.M * (B.g.is_complex ? 2 : 1);
+  const size_t vbytes = sizeof(float) * (size_t)nreal;
+  auto t1 = std::chrono::steady_clock::now();
+  gpe_status s = level_set_problem<double>(LP.d, gi, st);
+  if (s == GPE_OK) s = level_set_problem<float>(LP.f, gi, st);
+  if (s != GPE_OK) return s;
+  s = launch_convert<float, double>((const float*)((char*)B.x + vbytes * k), (double*)LP.d.xs[0], nreal, 1.0, st);
+  if (s == GPE_OK) s = normalise_slot0<double>(LP.d, st);
+  if (s != GPE_OK) return s;
+  LevelStats l2;
+  s = rn_run<double>(LP.d, P, 0, false, st, l2, 2.0 * r.mu, &LP.f);
+  if (s != GPE_OK) return s;
+  s = launch_convert<double, float>((const double*)LP.d.xk, (float*)psi[B.idx[k]], nreal, 1.0 / sqrt(B.g.hvol), st);
+  if (s != GPE_OK) return s;
   GPE_CUDA(cudaStreamSynchronize(st));
+  r.E = l2.F;
+  r.mu = 0.5 * l2.theta;
+  r.res = 0.5 * l2.res;
+  r.status = l2.converged ? GPE_OK : GPE_ENOCONV;
+  r.outer_f64 = l2.outer;
+  r.inner_f64 = l2.inner;
+  r.inner_f32 += l2.inner32;
+  r.nfe += l2.nfe;
+  r.ms_f64 = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t1).count();
+  return GPE_OK;
+}
+
+// One lane: instances from the pool until it is empty or an instance failed.
+static void refine_lane(RefinePool& pool, cudaStream_t st, const std::vector<GridHost>& gh, void* const* psi,
+                        const SolveParams& P, gpe_solve_report* reports) {
+  gpe_status s = GPE_OK;
+  std::string err;
+  try {
+    if (cudaSetDevice(pool.device) != cudaSuccess) s = fail(GPE_ECUDA, "cudaSetDevice in a refinement lane");
+    while (s == GPE_OK) {
+      BatchGroup* B = nullptr;
+      int k = 0;
+      std::unique_ptr<LevelPair> LP;
+      {
+        std::lock_guard<std::mutex> lk(pool.mu);
+        if (pool.status != GPE_OK || pool.next >= pool.todo.size()) break;
+        B = pool.todo[pool.next].first;
+        k = pool.todo[pool.next].second;
+        ++pool.next;
+        auto& v = pool.idle[B];
+        if (!v.empty()) {
+          LP = std::move(v.back());
+          v.pop_back();
+        }
+      }
+      if (!LP) {
+        LP.reset(new LevelPair());
+        s = LP->d.create(B->g);
+        if (s == GPE_OK) s = LP->f.create(B->g);
+      }
+      if (s == GPE_OK) s = refine_instance(*B, k, *LP, gh, psi, P, reports[B->idx[k]], st);
+      if (s != GPE_OK) cudaStreamSynchronize(st);   // before the pair may go
+      std::lock_guard<std::mutex> lk(pool.mu);
+      pool.idle[B].push_back(std::move(LP));
+    }
+    if (s != GPE_OK) err = gpe_last_error();
+  } catch (const std::bad_alloc&) {
+    s = GPE_ENOMEM;
+    err = "out of host memory in a refinement lane";
+  } catch (...) {
+    s = GPE_ECUDA;
+    err = "exception in a refinement lane";
+  }
+  if (s != GPE_OK) {
+    cudaStreamSynchronize(st);
+    std::lock_guard<std::mutex> lk(pool.mu);
+    if (pool.status == GPE_OK) {
+      pool.status = s;
+      pool.error = err;
+    }
+  }
+}
+
+// Every instance that has not reached res_tol, refined on up to REFINE_LANES
+// lanes; the calling thread is the first of them (and the only one where no
+// thread can be had).
+static gpe_status refine_batch(std::vector<std::unique_ptr<BatchGroup>>& groups, const std::vector<GridHost>& gh,
+                               void* const* psi, const SolveParams& P, gpe_solve_report* reports) {
+  RefinePool pool;
+  GPE_CUDA(cudaGetDevice(&pool.device));
+  std::vector<BatchGroup*> order;
+  for (auto& b : groups) order.push_back(b.get());
+  std::stable_sort(order.begin(), order.end(), [](const BatchGroup* a, const BatchGroup* b) {
+    return a->g.M * (a->g.is_complex + 1) > b->g.M * (b->g.is_complex + 1);
+  });
+  for (BatchGroup* B : order)
+    for (int k = 0; k < (int)B->idx.size(); ++k) {
+      const int st = reports[B->idx[k]].status;
+      if (st != GPE_ENONFINITE && st != GPE_OK) pool.todo.emplace_back(B, k);
+    }
+  if (pool.todo.empty()) return GPE_OK;
+  // private streams: the lanes capture CUDA graphs, which the caller's stream
+  // may not allow (the legacy default stream cannot be captured)
+  struct Lanes {
+    std::vector<cudaStream_t> st;
+    std::vector<std::thread> th;
+    ~Lanes() {
+      for (auto& t : th)
+        if (t.joinable()) t.join();
+      for (auto s : st) cudaStreamDestroy(s);
+    }
+  } lanes;
+  const unsigned cores = std::thread::hardware_concurrency();   // 0: unknown
+  const int n = (int)std::min<size_t>(cores ? std::min<unsigned>(REFINE_LANES, cores) : REFINE_LANES, pool.todo.size());
+  lanes.st.reserve(n);
+  lanes.th.reserve(n);
+  for (int i = 0; i < n; ++i) {
+    cudaStream_t s = nullptr;
+    GPE_CUDA(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
+    lanes.st.push_back(s);
+  }
+  for (int i = 1; i < n; ++i) {
+    const cudaStream_t s = lanes.st[i];
+    try {
+      lanes.th.emplace_back([&, s] { refine_lane(pool, s, gh, psi, P, reports); });
+    } catch (const std::system_error&) {
+      break;
+    }
+  }
+  refine_lane(pool, lanes.st[0], gh, psi, P, reports);
+  for (auto& t : lanes.th) t.join();
+  if (pool.status != GPE_OK) return fail(pool.status, pool.error);
   return GPE_OK;
 }
 
@@ -1460,10 +1594,31 @@ extern "C" gpe_status gpe_solve_batch(const gpe_problem* problems, int n, void* 
     }
     grp->idx.push_back(i);
   }
+  // the groups' stages on streams of their own, after the work queued on the
+  // caller's stream; the call ends when all of them have
+  struct Event {
+    cudaEvent_t e = nullptr;
+    ~Event() {
+      if (e) cudaEventDestroy(e);
+    }
+  } begin;
+  GPE_CUDA(cudaEventCreateWithFlags(&begin.e, cudaEventDisableTiming));
+  GPE_CUDA(cudaEventRecord(begin.e, st));
   for (auto& b : groups) {
-    gpe_status s = run_batch_group(*b, gh, psi, P, reports, st);
+    GPE_CUDA(cudaStreamCreateWithFlags(&b->st, cudaStreamNonBlocking));
+    GPE_CUDA(cudaStreamWaitEvent(b->st, begin.e, 0));
+    gpe_status s = queue_batch_group(*b, gh, psi, P);
     if (s != GPE_OK) return s;
   }
+  for (auto& b : groups) {
+    gpe_status s = finish_batch_group(*b, P, reports);
+    if (s != GPE_OK) return s;
+  }
+  if (P.refine) {
+    gpe_status s = refine_batch(groups, gh, psi, P, reports);
+    if (s != GPE_OK) return s;
+  }
+  GPE_CUDA(cudaStreamSynchronize(st));
   for (int i = 0; i < n; ++i)
     if (reports[i].status == GPE_ENONFINITE) return fail(GPE_ENONFINITE, "non-finite energy in a batched instance");
   return GPE_OK;
