@@ -233,7 +233,6 @@ __global__ void __launch_bounds__(FUSED_THREADS, fused_minb(LF)) k_fused2d(PassG
   constexpr unsigned FULL = 0xffffffffu;
   // a finished solver run (control block done) takes no tasks; the warps still
   // count themselves out below, so the counters are reset all the same
-  const bool idle = D.ctl && D.ctl->done;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* twx = reinterpret_cast<C*>(smem_raw);
   C* twy = twx + F;
@@ -244,6 +243,9 @@ __global__ void __launch_bounds__(FUSED_THREADS, fused_minb(LF)) k_fused2d(PassG
     twy[i] = reinterpret_cast<const C*>(FA.tw2y)[i];
   }
   __syncthreads();
+  pdl_next();
+  pdl_wait();
+  const bool idle = D.ctl && D.ctl->done;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int h = lane / TPL, j = lane & (TPL - 1);
   C* ex = exb + (warp * LPW + h) * FFT::P;
@@ -551,8 +553,7 @@ static gpe_status launch_fused2d_t(const GridHost& g, const GridDev<T>& d, const
   // (measured: 64 x 256^2 complex 87 -> 76 us per apply against once)
   FA.skew = (int)std::min<long long>(nb, (FUSED_SKEW * (long long)grid * wpc + FA.NY - 1) / FA.NY + 1);
   ProfScope ps(kernel_name("fused2d", 0, CPLX, EPI, g.M * nb), st);
-  k_fused2d<T, CPLX, EPI, LF, PK><<<grid, FUSED_THREADS, smem, st>>>(d.geom[0], d.geom[1], Df, FA);
-  GPE_CUDA(cudaGetLastError());
+  GPE_CUDA(launch_pdl(k_fused2d<T, CPLX, EPI, LF, PK>, grid, FUSED_THREADS, smem, st, d.geom[0], d.geom[1], Df, FA));
   return GPE_OK;
 }
 

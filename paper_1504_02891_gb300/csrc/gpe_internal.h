@@ -183,6 +183,7 @@ long long wait_limit(long long default_polls);
 // Instrumentation: launch counting and optional per-kernel CUDA-event timing.
 void instr_count(long long n);
 bool prof_enabled();
+bool stream_capturing(cudaStream_t st);
 struct ProfScope {
   int slot = -1;
   cudaStream_t st = nullptr;

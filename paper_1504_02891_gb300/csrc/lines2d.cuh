@@ -113,7 +113,6 @@ __global__ void __launch_bounds__(lines_y_threads<T>(LF)) k_lines_y(PassGeom<T> 
   constexpr int TPL = FFT::TPL;
   constexpr int CW = NT / TPL;
   constexpr int F = FFT::F;
-  if (D.ctl && D.ctl->done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   using X = typename FFT::X;
   typename FFT::Tw* tws = reinterpret_cast<typename FFT::Tw*>(smem_raw);
@@ -126,6 +125,9 @@ __global__ void __launch_bounds__(lines_y_threads<T>(LF)) k_lines_y(PassGeom<T> 
   const int cl = tid & (CW - 1), j = tid / CW;
   FFT fft;
   fft.init(j, tws);
+  pdl_next();
+  pdl_wait();
+  if (D.ctl && D.ctl->done) return;
   int par = 0;
   const int n0c = CPLX ? G.n0 : G.n0 >> 1;    // complex columns per row
   const C* xin = (const C*)D.x;
@@ -208,7 +210,6 @@ __global__ void __launch_bounds__(lines_x_threads<T>(LF), lines_x_minb<T>(LF)) k
   constexpr int NL = NT / TPL;
   constexpr int F = FFT::F;
   constexpr int NV = CPLX ? 8 : 16;           // values per thread and group (real: two rows)
-  if (D.ctl && D.ctl->done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   using X = typename FFT::X;
   typename FFT::Tw* tws = reinterpret_cast<typename FFT::Tw*>(smem_raw);
@@ -222,6 +223,9 @@ __global__ void __launch_bounds__(lines_x_threads<T>(LF), lines_x_minb<T>(LF)) k
   const int l = tid / TPL, j = tid & (TPL - 1);
   FFT fft;
   fft.init(j, tws);
+  pdl_next();
+  pdl_wait();
+  if (D.ctl && D.ctl->done) return;
   int par = 0;
   const int inst = blockIdx.x / tiles_per_inst;
   const int tile = blockIdx.x - inst * tiles_per_inst;
@@ -349,8 +353,7 @@ static gpe_status launch_lines_x(const GridDev<T>& d, const PassData<T>& Dx, int
   while (tiles > 1 && (long long)tiles * nbatch > d.max_blocks) tiles = (tiles + 1) / 2;
   if ((long long)tiles * nbatch > d.max_blocks) return fail(GPE_EINVAL, "reduction scratch too small");
   ProfScope ps(kernel_name("linesx", sizeof(T) == 8, CPLX, EPI, gx.M * nbatch), st);
-  k_lines_x<T, CPLX, EPI, LF0><<<nbatch * tiles, NTX, smem, st>>>(gx, Dx, tiles, groups);
-  GPE_CUDA(cudaGetLastError());
+  GPE_CUDA(launch_pdl(k_lines_x<T, CPLX, EPI, LF0>, nbatch * tiles, NTX, smem, st, gx, Dx, tiles, groups));
   return GPE_OK;
 }
 
@@ -381,8 +384,7 @@ static gpe_status launch_lines2d_t(const GridDev<T>& d, const PassData<T>& D, in
     const int total = nbatch * colgroups;
     const int grid = std::min(total, tuned_waves(1, sizeof(T) == 8, CPLX, gx.n0, gx.n1, nbatch) * sh.occ * num_sms());
     ProfScope ps(kernel_name("linesy", sizeof(T) == 8, CPLX, EPI_ACC, gx.M * nbatch), st);
-    k_lines_y<T, CPLX, LF1><<<grid, YT, smem, st>>>(gy, Dy, colgroups, total);
-    GPE_CUDA(cudaGetLastError());
+    GPE_CUDA(launch_pdl(k_lines_y<T, CPLX, LF1>, grid, YT, smem, st, gy, Dy, colgroups, total));
   }
   // x pass with the epilogue
   {

@@ -75,7 +75,6 @@ __global__ void __launch_bounds__(axs_threads<T>(LF)) k_axis_s(PassGeom<T> G, Pa
   using V = typename VT<T, KIND == LK_CPLX>::V;
   constexpr int F = FFT::F, TPL = FFT::TPL, CW = axs_cw<T>(LF), NT = axs_threads<T>(LF);
   constexpr int NP = KIND == LK_SINE ? 4 : 8;    // data points per thread and line
-  if (D.ctl && D.ctl->done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   typename FFT::Tw* tws = reinterpret_cast<typename FFT::Tw*>(smem_raw);
   X* xb = reinterpret_cast<X*>(tws + F);         // [2][F][CW]
@@ -83,6 +82,12 @@ __global__ void __launch_bounds__(axs_threads<T>(LF)) k_axis_s(PassGeom<T> G, Pa
   const int tid = threadIdx.x;
   const int cl = tid & (CW - 1), j = tid / CW;
   const int plane = blockIdx.x / tiles, tile = blockIdx.x - plane * tiles;
+  load_table(tws, line_table<FFT>(G), F);
+  FFT fft;
+  fft.init(j, tws);
+  pdl_next();
+  pdl_wait();
+  if (D.ctl && D.ctl->done) return;
   const V* x0 = (const V*)D.x;
   const V* x1 = (const V*)D.xsub;
   V* yst = nullptr;
@@ -154,9 +159,6 @@ __global__ void __launch_bounds__(axs_threads<T>(LF)) k_axis_s(PassGeom<T> G, Pa
       }
     }
   }
-  load_table(tws, line_table<FFT>(G), F);
-  FFT fft;
-  fft.init(j, tws);
   int par = 0;
   ExCols<X, CW> ex{xb + cl, F * CW, s_red};
   if constexpr (KIND == LK_SINE) mirror_odd<T, LF>(v, ex, par, j);
@@ -192,7 +194,6 @@ __global__ void __launch_bounds__(axx_threads<T>(LF), axx_minb<T>(LF)) k_axis_x(
   constexpr int NP = KIND == LK_SINE ? 4 : 8;    // data points per thread and row
   constexpr int NV = CPLX ? NP : 2 * NP;         // values per thread
   constexpr bool REGS = sizeof(T) == 4;          // epilogue operands in registers
-  if (D.ctl && D.ctl->done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   typename FFT::Tw* tws = reinterpret_cast<typename FFT::Tw*>(smem_raw);
   X* xb = reinterpret_cast<X*>(tws + F);         // [2][NL][P]
@@ -204,6 +205,9 @@ __global__ void __launch_bounds__(axx_threads<T>(LF), axx_minb<T>(LF)) k_axis_x(
   const int l = tid / TPL, j = tid & (TPL - 1);
   FFT fft;
   fft.init(j, tws);
+  pdl_next();
+  pdl_wait();
+  if (D.ctl && D.ctl->done) return;
   int par = 0;
   const int inst = blockIdx.x / tiles_per_inst;
   const int tile = blockIdx.x - inst * tiles_per_inst;
@@ -339,8 +343,7 @@ static gpe_status launch_axis_s_t(const GridDev<T>& d, int axis, const PassData<
   const int cols = KIND == LK_CPLX ? CW : 2 * CW;
   const int tiles = (width + cols - 1) / cols;
   ProfScope ps(kernel_name("axis_s", sizeof(T) == 8, KIND == LK_CPLX, EPI_ACC, G.M * nbatch), st);
-  k_axis_s<T, KIND, LF><<<planes * tiles, NT, smem, st>>>(G, D, width, tiles);
-  GPE_CUDA(cudaGetLastError());
+  GPE_CUDA(launch_pdl(k_axis_s<T, KIND, LF>, planes * tiles, NT, smem, st, G, D, width, tiles));
   return GPE_OK;
 }
 
@@ -363,8 +366,7 @@ static gpe_status launch_axis_x_t(const GridDev<T>& d, const PassData<T>& D, int
   const int tiles = (int)std::max<long long>(1, std::min<long long>(groups, std::max<long long>(cap / nbatch, 1)));
   if ((long long)tiles * nbatch > d.max_blocks) return fail(GPE_EINVAL, "reduction scratch too small");
   ProfScope ps(kernel_name("axis_x", sizeof(T) == 8, KIND == LK_CPLX, EPI, G.M * nbatch), st);
-  k_axis_x<T, KIND, EPI, LF><<<nbatch * tiles, NT, smem, st>>>(G, D, tiles, groups);
-  GPE_CUDA(cudaGetLastError());
+  GPE_CUDA(launch_pdl(k_axis_x<T, KIND, EPI, LF>, nbatch * tiles, NT, smem, st, G, D, tiles, groups));
   return GPE_OK;
 }
 

@@ -719,6 +719,37 @@ static __device__ void rn_control(RNCtl* c, const double* r) {
   c->delta = fmin(fmax(nd, c->delta_min), c->delta_max);
 }
 
+// ----------------------------------------------------------------- dependent launches
+// The kernels of one operator application follow one another on a stream, each
+// a few microseconds long, and a launch costs one to two.  They are launched
+// with programmatic stream serialisation: a kernel may be made resident while
+// the one before it drains, loads its constant tables, and waits
+// (griddepcontrol.wait) for that kernel's completion and memory before it
+// touches anything else.  Every CTA of every such kernel executes the wait
+// before it can return, so completion is transitive along the stream.  Launches
+// being captured keep plain edges: the solver's graphs of 16 iterations ran 2%
+// slower with programmatic ones (64^3: 14.9 against 14.6 ms a solve).  Measured:
+// 127^3 Hessian-vector float32 59 -> 50 us, 64^3 -> 128^3 transfer 32 -> 24 us,
+// 512^2 complex128 Hessian-vector 36.9 -> 34.5 us.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Let the next kernel be made resident (once every CTA has got here or ended).
+__device__ __forceinline__ void pdl_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... P, typename... A>
+static cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = stream_capturing(st) ? 0 : 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // ----------------------------------------------------------------- coherent loads
 // Inside a persistent launch, data written by other CTAs during the same launch
 // must bypass the (non-coherent) L1: ld.global.cg.
@@ -1278,6 +1309,8 @@ __global__ void __launch_bounds__(NTHREADS) k_fd(FDGeom G, const T* __restrict__
 template <typename T, bool CPLX>
 __global__ void k_step(void* const* xs, void* const* gs, const Alg1Ctl* c, long long n, const void* xkv) {
   using V = typename VT<T, CPLX>::V;
+  pdl_next();
+  pdl_wait();
   if (c->done) return;
   const V* X = (const V*)xs[c->cur];
   const V* Gv = (const V*)gs[c->cur];
@@ -1345,6 +1378,8 @@ __global__ void __launch_bounds__(NTHREADS) k_moments(const void* xv, const void
                                                       MomentCoef mc) {
   using V = typename VT<T, CPLX>::V;
   using P = Pack<V, W>;
+  pdl_next();
+  pdl_wait();
   const int inst = blockIdx.x / tiles;
   const int tb = blockIdx.x - inst * tiles;
   const P* x = reinterpret_cast<const P*>((const V*)xv + inst * M);
@@ -1397,6 +1432,8 @@ __global__ void __launch_bounds__(NTHREADS) k_axpby(const void* xv, const void* 
   using V = typename VT<T, CPLX>::V;
   using P = Pack<V, W>;
   const long long n = M / W;
+  pdl_next();
+  pdl_wait();
   for (int b = blockIdx.y; b < nbatch; b += gridDim.y) {
     const P* x = reinterpret_cast<const P*>((const V*)xv + b * M);
     const P* g = gv ? reinterpret_cast<const P*>((const V*)gv + b * M) : nullptr;
@@ -1428,9 +1465,9 @@ static void run_moments(const void* x, const void* g, long long M, int nbatch, i
   using V = typename VT<T, CPLX>::V;
   constexpr int W = (int)(16 / sizeof(V));
   if (pack_width(sizeof(V), M, x, g, nullptr) > 1)
-    k_moments<T, CPLX, W><<<tiles * nbatch, NTHREADS, 0, st>>>(x, g, M, tiles, partials, results, ticket, mc);
+    launch_pdl(k_moments<T, CPLX, W>, tiles * nbatch, NTHREADS, 0, st, x, g, M, tiles, partials, results, ticket, mc);
   else
-    k_moments<T, CPLX, 1><<<tiles * nbatch, NTHREADS, 0, st>>>(x, g, M, tiles, partials, results, ticket, mc);
+    launch_pdl(k_moments<T, CPLX, 1>, tiles * nbatch, NTHREADS, 0, st, x, g, M, tiles, partials, results, ticket, mc);
 }
 template <typename T, bool CPLX>
 static void run_axpby(const void* x, const void* g, const double* coef, int stride, long long M, int nbatch, void* out,
@@ -1442,8 +1479,8 @@ static void run_axpby(const void* x, const void* g, const double* coef, int stri
   const int gy = std::min(nbatch, 65535);
   const long long full = (M / w + NTHREADS - 1) / NTHREADS;
   const int gx = (int)std::max<long long>(1, std::min<long long>(full, std::max(1, 152 * 8 / gy)));
-  if (w > 1) k_axpby<T, CPLX, W><<<dim3(gx, gy), NTHREADS, 0, st>>>(x, g, coef, stride, M, nbatch, out);
-  else k_axpby<T, CPLX, 1><<<dim3(gx, gy), NTHREADS, 0, st>>>(x, g, coef, stride, M, nbatch, out);
+  if (w > 1) launch_pdl(k_axpby<T, CPLX, W>, dim3(gx, gy), NTHREADS, 0, st, x, g, coef, stride, M, nbatch, out);
+  else launch_pdl(k_axpby<T, CPLX, 1>, dim3(gx, gy), NTHREADS, 0, st, x, g, coef, stride, M, nbatch, out);
 }
 
 // Shifted subproblem inputs in float32: X^k and P_k = G_k - theta_k X^k

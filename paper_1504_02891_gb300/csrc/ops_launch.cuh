@@ -315,8 +315,8 @@ template <typename T>
 gpe_status launch_step(void* const* xs, void* const* gs, const Alg1Ctl* ctl, long long n, int cplx, cudaStream_t st,
                        const void* xk) {
   ProfScope ps(kernel_name("step", sizeof(T) == 8, cplx, -1, n), st);
-  if (cplx) k_step<T, true><<<ew_blocks(n), NTHREADS, 0, st>>>(xs, gs, ctl, n, xk);
-  else k_step<T, false><<<ew_blocks(n), NTHREADS, 0, st>>>(xs, gs, ctl, n, xk);
+  if (cplx) launch_pdl(k_step<T, true>, ew_blocks(n), NTHREADS, 0, st, xs, gs, ctl, n, xk);
+  else launch_pdl(k_step<T, false>, ew_blocks(n), NTHREADS, 0, st, xs, gs, ctl, n, xk);
   GPE_CUDA(cudaGetLastError());
   return GPE_OK;
 }

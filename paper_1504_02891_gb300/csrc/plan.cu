@@ -37,7 +37,7 @@ static std::vector<ProfRec> g_recs;
 void instr_count(long long n) { g_launches += n; }
 bool prof_enabled() { return g_prof.load(); }
 
-static bool capturing(cudaStream_t st) {
+bool stream_capturing(cudaStream_t st) {
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) return false;
   return cs != cudaStreamCaptureStatusNone;
@@ -45,7 +45,7 @@ static bool capturing(cudaStream_t st) {
 
 ProfScope::ProfScope(const char* name, cudaStream_t s) {
   st = s;
-  if (capturing(s)) return;   // counted when the graph is launched
+  if (stream_capturing(s)) return;   // counted when the graph is launched
   g_launches += 1;
   if (!g_prof.load()) return;
   ProfRec r;

@@ -80,6 +80,11 @@ __global__ void __launch_bounds__(axs_threads<T>(LF)) k_prolong_s(ProlongArgs<T>
   const int c0 = KIND == LK_CPLX ? tile * CW + cl : (KIND == LK_REAL ? 2 * (tile * CW + cl) : 2 * tile * CW + cl);
   const int c1 = KIND == LK_REAL ? c0 + 1 : c0 + CW;
   const bool in0 = c0 < width, in1 = KIND != LK_CPLX && c1 < width;
+  load_table(tws, line_table<FFT>(G), F);
+  FFT fft;
+  fft.init(j, tws);
+  pdl_next();
+  pdl_wait();
   const V* in = (const V*)A.in + (long long)plane * G.len * width;
   const int flen = KIND == LK_SINE ? 2 * G.len + 1 : 2 * G.len;
   V* out = (V*)A.out + (long long)plane * flen * width;
@@ -97,9 +102,6 @@ __global__ void __launch_bounds__(axs_threads<T>(LF)) k_prolong_s(ProlongArgs<T>
     }
     x[s] = v[s];
   }
-  load_table(tws, line_table<FFT>(G), F);
-  FFT fft;
-  fft.init(j, tws);
   int par = 0;
   ExCols<X, CW> ex{xb + cl, F * CW, s_red};
   if constexpr (KIND == LK_SINE) mirror_odd<T, LF>(v, ex, par, j);
@@ -141,6 +143,11 @@ __global__ void __launch_bounds__(axx_threads<T>(LF)) k_prolong_x(ProlongArgs<T>
   const int rows = (int)(G.M / G.len);
   const int r0 = CPLX ? grp * NL + l : 2 * (grp * NL + l);
   const bool in0 = r0 < rows, in1 = !CPLX && r0 + 1 < rows;
+  load_table(tws, line_table<FFT>(G), F);
+  FFT fft;
+  fft.init(j, tws);
+  pdl_next();
+  pdl_wait();
   const V* in = (const V*)A.in + (long long)inst * G.M + (long long)r0 * G.len;
   const int flen = KIND == LK_SINE ? 2 * G.len + 1 : 2 * G.len;
   V* out = (V*)A.out + ((long long)inst * rows + r0) * flen;
@@ -158,9 +165,6 @@ __global__ void __launch_bounds__(axx_threads<T>(LF)) k_prolong_x(ProlongArgs<T>
     }
     x[s] = v[s];
   }
-  load_table(tws, line_table<FFT>(G), F);
-  FFT fft;
-  fft.init(j, tws);
   int par = 0;
   ExRow<X, FFT::P> ex{xb + l * FFT::P, NL * FFT::P, 1 + l, TPL, s_red};
   if constexpr (KIND == LK_SINE) mirror_odd<T, LF>(v, ex, par, j);
@@ -192,7 +196,7 @@ static gpe_status launch_prolong_line_t(int axis, ProlongArgs<T> A, int nbatch, 
     GPE_CUDA(allowed);
     const long long rows = G.M / G.len, lines = KIND == LK_CPLX ? rows : (rows + 1) / 2;
     A.tiles = (int)((lines + NL - 1) / NL);
-    k_prolong_x<T, KIND, LF><<<nbatch * A.tiles, NT, smem, st>>>(A);
+    GPE_CUDA(launch_pdl(k_prolong_x<T, KIND, LF>, nbatch * A.tiles, NT, smem, st, A));
   } else {
     constexpr int CW = axs_cw<T>(LF), NT = axs_threads<T>(LF);
     const size_t smem = (size_t)FFT::F * sizeof(typename FFT::Tw) + 2 * (size_t)FFT::F * CW * sizeof(typename FFT::X);
@@ -202,9 +206,8 @@ static gpe_status launch_prolong_line_t(int axis, ProlongArgs<T> A, int nbatch, 
     A.planes_per_inst = axis == 1 ? G.n2 : 1;
     const int cols = KIND == LK_CPLX ? CW : 2 * CW;
     A.tiles = (A.width + cols - 1) / cols;
-    k_prolong_s<T, KIND, LF><<<nbatch * A.planes_per_inst * A.tiles, NT, smem, st>>>(A);
+    GPE_CUDA(launch_pdl(k_prolong_s<T, KIND, LF>, nbatch * A.planes_per_inst * A.tiles, NT, smem, st, A));
   }
-  GPE_CUDA(cudaGetLastError());
   return GPE_OK;
 }
 
