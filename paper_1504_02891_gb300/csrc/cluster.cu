@@ -68,14 +68,10 @@ __device__ __forceinline__ void dsmem_st2(unsigned addr, float2 v) {
   asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};\n" ::"r"(addr), "f"(v.x), "f"(v.y) : "memory");
 }
 
-// The CTA's partial sums of the NQ quantities into out[0..NQ) (float pairs).
-// Within a warp a reduce-scatter: at offsets 16, 8, 4, 2 a lane keeps one half
-// of its quantities (chosen by its lane bit) and adds its partner's copy of
-// that half, so after four steps lane l holds quantity (l >> 1) & 15 summed
-// over the 16 lanes of its parity, and offset 1 adds the other parity: 16
-// merges and 32 shuffles per lane instead of a 5-level tree per quantity.  The
-// max-norm slot is reduced by its own shuffle tree.  Then NQ threads fold the
-// warps' sums in warp order.  Every CTA and every run folds in the same order.
+// The CTA's partial sums of the NQ quantities into out[0..NQ) (float pairs):
+// a warp reduce-scatter, the max-norm slot by its own shuffle tree, then NQ
+// threads fold the warps' sums in warp order.  Every CTA and every run folds in
+// the same order.
 __device__ __forceinline__ void cluster_block_partial(const DF (&acc)[NQ], float amax2, double* out) {
   static_assert(NQ <= 16, "16 reduce-scatter slots");
   __shared__ DF red[NTHREADS / 32][16];
@@ -86,33 +82,7 @@ __device__ __forceinline__ void cluster_block_partial(const DF (&acc)[NQ], float
     if (q < NQ && q != Q_MAX) v[q] = acc[q];
     else acc_zero(v[q]);
   }
-#pragma unroll
-  for (int o = 16, H = 8; o >= 2; o >>= 1, H >>= 1) {
-    const bool up = (lane & o) != 0;
-#pragma unroll
-    for (int i = 0; i < H; ++i) {
-      const DF keep = up ? v[i + H] : v[i];
-      const DF send = up ? v[i] : v[i + H];
-      DF w;
-      w.hi = __shfl_xor_sync(0xffffffffu, send.hi, o);
-      w.lo = __shfl_xor_sync(0xffffffffu, send.lo, o);
-      v[i] = keep;
-      acc_merge(v[i], w);
-    }
-  }
-  {
-    DF w;
-    w.hi = __shfl_xor_sync(0xffffffffu, v[0].hi, 1);
-    w.lo = __shfl_xor_sync(0xffffffffu, v[0].lo, 1);
-    // the two parities in a fixed order (even lane's sum first)
-    if (lane & 1) {
-      DF t = w;
-      acc_merge(t, v[0]);
-      v[0] = t;
-    } else {
-      acc_merge(v[0], w);
-    }
-  }
+  const DF r = warp_reduce_scatter(v);
   float m = sqrtf(amax2);
   for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
   const int q = (lane >> 1) & 15;
@@ -121,7 +91,7 @@ __device__ __forceinline__ void cluster_block_partial(const DF (&acc)[NQ], float
       red[warp][q].hi = m;
       red[warp][q].lo = 0.f;
     } else {
-      red[warp][q] = v[0];
+      red[warp][q] = r;
     }
   }
   __syncthreads();

@@ -90,7 +90,7 @@ struct Scratch {
   double* partials = nullptr;
   double* results = nullptr;     // [nbatch][NQ]
   double* coef = nullptr;        // [nbatch][4]
-  unsigned int* ticket = nullptr;   // [nbatch], zero between launches
+  unsigned int* ticket = nullptr;   // fold_tickets(cap_blocks, nbatch), zero between launches
   // [nbatch][NQ] in pinned host memory: the energy entry points have the
   // reductions write their sums here (no copy to wait for), and the fused
   // kernel's expired-wait flag behind them
@@ -139,6 +139,9 @@ gpe_status launch_add_f32_to_f64(const double* xk, const float* d, double* z, lo
 template <typename T>
 gpe_status apply_op(const GridHost& g, const GridDev<T>& d, PassData<T> D, int epi, void* acc, bool step_first,
                     cudaStream_t st);
+
+// Whether apply_op with EPI_WS and step_first forms the difference-form step.
+template <typename T> bool shifted_step_ok(const GridHost& g);
 
 template <typename T>
 gpe_status persist_config(const GridHost& g, const GridDev<T>& d, int epi, int* grid, size_t* smem);

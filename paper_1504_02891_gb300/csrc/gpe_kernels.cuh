@@ -198,7 +198,8 @@ struct PassData {
   void* const* gs;      // 3 G slots
   Alg1Ctl* ctl;         // non-null in solver mode
   RNCtl* rn;            // ratio pass
-  int step_on_load;     // Y = s(a X_cur + b G_cur) formed on load, stored to xs[trial]
+  int step_on_load;     // 1: Y = s(a X_cur + b G_cur) formed on load, stored to xs[trial];
+                        // 2: the difference form D+ = (a - 1) X^k + a D + b G^ (X^k = base)
   int use_slots;        // x = xs[trial], out = gs[trial] (final), xc/gc from slots
   // pointwise data
   const T* V;
@@ -210,7 +211,7 @@ struct PassData {
   // reductions
   double* partials;     // [gridDim.x][NQ]
   double* results;      // [nbatch][NQ]
-  unsigned int* ticket; // [nbatch]
+  unsigned int* ticket; // per instance, then per group of CTAs (see reduce_partials)
   double* err;          // fused kernel: set to 1 when a task wait gave up (may be null)
   int nq;               // active slots (0: none)
   int control;          // 0: none, 1: Algorithm 1 control, 2: ratio control

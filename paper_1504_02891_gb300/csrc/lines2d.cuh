@@ -133,7 +133,8 @@ __global__ void __launch_bounds__(lines_y_threads<T>(LF)) k_lines_y(PassGeom<T> 
   const C* xin = (const C*)D.x;
   const C* src1 = (const C*)D.xsub;
   C* yst = nullptr;
-  T sa = 0, sb = 0;
+  const C* xk = nullptr;
+  T sa = 0, sb = 0, sk = 0;
   if (D.use_slots) {
     const Alg1Ctl* c = D.ctl;
     xin = (const C*)D.xs[c->trial];
@@ -143,6 +144,12 @@ __global__ void __launch_bounds__(lines_y_threads<T>(LF)) k_lines_y(PassGeom<T> 
       src1 = (const C*)D.gs[c->cur];
       sa = (T)(c->s * c->a);
       sb = (T)(c->s * c->b);
+      if (D.step_on_load == 2) {
+        xk = (const C*)D.base;
+        sk = (T)c->am1;
+        sa = (T)c->a;
+        sb = (T)c->b;
+      }
     }
   }
   C* out = (C*)D.out;
@@ -175,7 +182,8 @@ __global__ void __launch_bounds__(lines_y_threads<T>(LF)) k_lines_y(PassGeom<T> 
       C a = pf0[s * NT + tid];
       if (src1) {
         const C b = pf1[s * NT + tid];
-        a = yst ? sa * a + sb * b : a - b;
+        if (xk) a = sk * __ldg(xk + base + (long long)(j + s * TPL) * n0c) + sa * a + sb * b;
+        else a = yst ? sa * a + sb * b : a - b;
         if (yst) yst[base + (long long)(j + s * TPL) * n0c] = a;
       }
       v[s] = a;
@@ -329,7 +337,7 @@ __global__ void __launch_bounds__(lines_x_threads<T>(LF), lines_x_minb<T>(LF)) k
     b ^= 1;
   }
   if (EPI == EPI_HESS || D.nq == 0) return;
-  if (reduce_partials(acc, amax, D.nq, D.partials, D.results, D.ticket, tiles_per_inst)) run_control<T>(D);
+  run_control<T>(D, reduce_partials(acc, amax, D.nq, D.partials, D.results, D.ticket, tiles_per_inst));
 }
 
 template <typename T, bool CPLX, int EPI, int LF0>
@@ -373,7 +381,7 @@ static gpe_status launch_lines2d_t(const GridDev<T>& d, const PassData<T>& D, in
   // y pass (first: it also forms the trial point)
   {
     PassData<T> Dy = D;
-    Dy.step_on_load = step_first ? 1 : 0;
+    Dy.step_on_load = step_first ? (EPI == EPI_WS ? 2 : 1) : 0;
     Dy.acc_in = nullptr;
     Dy.out = acc;
     Dy.nq = 0;
@@ -411,6 +419,8 @@ static bool lines2d_ok(const GridHost& g) {
   return n0c % cw == 0 && lines % nl == 0;
 }
 
+template <typename T> bool lines2d_takes(const GridHost& g) { return lines2d_ok<T>(g) && lines2d_enabled(); }
+
 template <typename T, bool CPLX, int EPI, int LF0>
 static gpe_status lines2d_dispatch1(const GridDev<T>& d, const PassData<T>& D, int nbatch, void* acc, bool step_first,
                                     int lf1, cudaStream_t st) {
@@ -444,7 +454,9 @@ gpe_status launch_lines2d(const GridHost& g, const GridDev<T>& d, const PassData
   gpe_status s;
   if constexpr (std::is_same<T, float>::value) {
     const int path = operator_path();
-    const bool fused = path == 1 || (path == 0 && tuned_fused(g.is_complex, g.ext[0], g.nbatch));
+    // (the fused kernel does not form the difference-form step)
+    const bool fused = !(step_first && epi == EPI_WS) &&
+                       (path == 1 || (path == 0 && tuned_fused(g.is_complex, g.ext[0], g.nbatch)));
     if (fused2d_ok<T>(g) && fused && fused2d_enabled() && lines2d_enabled()) {
 #define GPE_F2D_CASE(E)                                                                    \
   case E:                                                                                  \

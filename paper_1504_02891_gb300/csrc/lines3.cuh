@@ -91,7 +91,8 @@ __global__ void __launch_bounds__(axs_threads<T>(LF)) k_axis_s(PassGeom<T> G, Pa
   const V* x0 = (const V*)D.x;
   const V* x1 = (const V*)D.xsub;
   V* yst = nullptr;
-  T sa = 0, sb = 0;
+  const V* xk = nullptr;
+  T sa = 0, sb = 0, sk = 0;
   if (D.use_slots) {
     const Alg1Ctl* c = D.ctl;
     x0 = (const V*)D.xs[c->trial];
@@ -101,6 +102,12 @@ __global__ void __launch_bounds__(axs_threads<T>(LF)) k_axis_s(PassGeom<T> G, Pa
       x1 = (const V*)D.gs[c->cur];
       sa = (T)(c->s * c->a);
       sb = (T)(c->s * c->b);
+      if (D.step_on_load == 2) {
+        xk = (const V*)D.base;
+        sk = (T)c->am1;
+        sa = (T)c->a;
+        sb = (T)c->b;
+      }
     }
   }
   const V* acc = (const V*)D.acc_in;
@@ -126,8 +133,13 @@ __global__ void __launch_bounds__(axs_threads<T>(LF)) k_axis_s(PassGeom<T> G, Pa
       if (in1) q = x0[off(s, c1)];
       if (x1) {
         const V p1 = in0 ? x1[off(s, c0)] : vzero<V>(), q1 = in1 ? x1[off(s, c1)] : vzero<V>();
-        p = yst ? sa * p + sb * p1 : p - p1;
-        q = yst ? sa * q + sb * q1 : q - q1;
+        if (xk) {
+          p = (in0 ? sk * xk[off(s, c0)] : vzero<V>()) + sa * p + sb * p1;
+          q = (in1 ? sk * xk[off(s, c1)] : vzero<V>()) + sa * q + sb * q1;
+        } else {
+          p = yst ? sa * p + sb * p1 : p - p1;
+          q = yst ? sa * q + sb * q1 : q - q1;
+        }
       }
     }
     if constexpr (KIND == LK_CPLX) {
@@ -214,7 +226,8 @@ __global__ void __launch_bounds__(axx_threads<T>(LF), axx_minb<T>(LF)) k_axis_x(
   const V* xin = (const V*)D.x;
   const V* xsub = (const V*)D.xsub;
   V* yst = nullptr;
-  T sa = 0, sb = 0;
+  const V* xk = nullptr;
+  T sa = 0, sb = 0, sk = 0;
   if (D.use_slots) {
     const Alg1Ctl* c = D.ctl;
     xin = (const V*)D.xs[c->trial];
@@ -224,6 +237,12 @@ __global__ void __launch_bounds__(axx_threads<T>(LF), axx_minb<T>(LF)) k_axis_x(
       xsub = (const V*)D.gs[c->cur];
       sa = (T)(c->s * c->a);
       sb = (T)(c->s * c->b);
+      if (D.step_on_load == 2) {
+        xk = (const V*)D.base;
+        sk = (T)c->am1;
+        sa = (T)c->a;
+        sb = (T)c->b;
+      }
     }
   }
   const V* accin = (const V*)D.acc_in;
@@ -260,7 +279,8 @@ __global__ void __launch_bounds__(axx_threads<T>(LF), axx_minb<T>(LF)) k_axis_x(
         xv[q] = xin[ibase + at(q)];
         if (xsub) {
           const V b = xsub[ibase + at(q)];
-          xv[q] = yst ? sa * xv[q] + sb * b : xv[q] - b;
+          if (xk) xv[q] = sk * xk[ibase + at(q)] + sa * xv[q] + sb * b;
+          else xv[q] = yst ? sa * xv[q] + sb * b : xv[q] - b;
         }
       }
     }
@@ -324,7 +344,7 @@ __global__ void __launch_bounds__(axx_threads<T>(LF), axx_minb<T>(LF)) k_axis_x(
     }
   }
   if (EPI == EPI_HESS || D.nq == 0) return;
-  if (reduce_partials(acc, amax, D.nq, D.partials, D.results, D.ticket, tiles_per_inst)) run_control<T>(D);
+  run_control<T>(D, reduce_partials(acc, amax, D.nq, D.partials, D.results, D.ticket, tiles_per_inst));
 }
 
 static inline int line_kind(const GridHost& g) {

@@ -30,10 +30,13 @@ constexpr size_t NOALLOC_PARTIALS = (size_t)NOALLOC_MAX_BLOCKS * gpe::NQ;   // d
 constexpr size_t NOALLOC_RESULTS = (size_t)NOALLOC_MAX_BATCH * gpe::NQ;     // doubles
 constexpr size_t NOALLOC_COEF = (size_t)NOALLOC_MAX_BATCH * 2;              // doubles
 constexpr size_t NOALLOC_BYTES = 512 * 1024;
-static_assert((NOALLOC_PARTIALS + NOALLOC_RESULTS + NOALLOC_COEF) * sizeof(double) + 256 <= NOALLOC_BYTES,
+constexpr size_t NOALLOC_TICKETS = 2 * NOALLOC_MAX_BATCH + NOALLOC_MAX_BLOCKS / gpe::FOLD_GROUP + 1;
+static_assert((NOALLOC_PARTIALS + NOALLOC_RESULTS + NOALLOC_COEF) * sizeof(double) +
+                      NOALLOC_TICKETS * sizeof(unsigned int) <=
+                  NOALLOC_BYTES,
               "scratch layout exceeds the array");
 
-// partials | results | coef | tickets (unsigned int per instance), each 256-byte aligned
+// partials | results | coef | tickets (unsigned int)
 static __device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_BYTES];
 
 std::mutex g_mu;
@@ -112,7 +115,7 @@ gpe_status run(const void* psi, const void* hpsi, long long M, int nbatch, doubl
   double* coef = results + NOALLOC_RESULTS;
   unsigned int* ticket = reinterpret_cast<unsigned int*>(coef + NOALLOC_COEF);
   // the array keeps the previous call's contents: the tickets must start at zero
-  cudaError_t e = cudaMemsetAsync(ticket, 0, sizeof(unsigned int) * NOALLOC_MAX_BATCH, st);
+  cudaError_t e = cudaMemsetAsync(ticket, 0, sizeof(unsigned int) * NOALLOC_TICKETS, st);
   if (e != cudaSuccess) return gpe::cuda_fail(e, "cudaMemsetAsync(ticket)");
   const gpe::MomentCoef mc{1, h, tau, coef};
   gpe::run_moments<T, CPLX>(psi, hpsi, M, nbatch, tiles, partials, results, ticket, mc, st);

@@ -351,48 +351,94 @@ __device__ __forceinline__ void cp_async_wait_all() {
 // the float64 pipe until its final NQ values.
 __device__ __forceinline__ void df_max(DF& a, const DF& b) { a.hi = fmaxf(a.hi, b.hi); }
 
-// Reduce the per-thread sums acc[0..nq) and the max slot over the block and
-// write this CTA's partials to out[0..NQ) (slots >= nq other than Q_MAX as 0).
-// Ends with a barrier.
+// The sums of a warp: at offsets 16, 8, 4, 2 a lane keeps one half of its
+// quantities (chosen by its lane bit) and adds its partner's copy of that half,
+// so after four steps lane l holds quantity (l >> 1) & 15 summed over the 16
+// lanes of its parity, and offset 1 adds the other parity: 16 merges and 32
+// shuffles per lane instead of a 5-level tree per quantity (75 merges).  The
+// float64 trees were a quarter of the float64 instructions of whole kernels.
+__device__ __forceinline__ DF shfl_xor(const DF& a, int o) {
+  DF r;
+  r.hi = __shfl_xor_sync(0xffffffffu, a.hi, o);
+  r.lo = __shfl_xor_sync(0xffffffffu, a.lo, o);
+  return r;
+}
+__device__ __forceinline__ double shfl_xor(double a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
+template <typename A> __device__ __forceinline__ A warp_reduce_scatter(A (&v)[16]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 16, H = 8; o >= 2; o >>= 1, H >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int i = 0; i < H; ++i) {
+      const A keep = up ? v[i + H] : v[i];
+      const A send = up ? v[i] : v[i + H];
+      const A w = shfl_xor(send, o);
+      v[i] = keep;
+      acc_merge(v[i], w);
+    }
+  }
+  // the two parities in a fixed order (even lane's sum first)
+  const A w = shfl_xor(v[0], 1);
+  A r = (lane & 1) ? w : v[0];
+  acc_merge(r, (lane & 1) ? v[0] : w);
+  return r;
+}
+__device__ __forceinline__ void acc_max(DF& a, const DF& b) { a.hi = fmaxf(a.hi, b.hi); }
+__device__ __forceinline__ void acc_max(double& a, double b) { a = fmax(a, b); }
+
+// Reduce the per-thread sums acc[0..nq) over the block and write this CTA's
+// partials to out[0..NQ); the other slots are 0.  Slot Q_MAX, the largest |.|
+// (amax2: its square), is reduced when all NQ slots are asked for.  Ends with
+// a barrier.
 template <typename A, typename M>
 static __device__ void block_partial(A (&acc)[NQ], M amax2, int nq, double* out) {
-  // amax2 is the largest |.|^2 of the CTA's points; a float32 run takes the
-  // root in float32 (correctly rounded, the same value as the float64 root
-  // rounded to float32; a float64 root costs ~0.3 us and the FP64 pipe)
-  constexpr bool F32ACC = sizeof(A) == sizeof(DF) && !std::is_same<A, double>::value;
-  const double acc_max = F32ACC ? 0.0 : sqrt((double)amax2);
-  const float acc_max_f = F32ACC ? sqrtf((float)amax2) : 0.f;
-  __shared__ A red[NTHREADS / 32][NQ];
+  constexpr bool F32ACC = !std::is_same<A, double>::value;
+  __shared__ A red[NTHREADS / 32][16];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nw = blockDim.x >> 5;
+  if (nq < NQ) {
 #pragma unroll
-  for (int q = 0; q < NQ; ++q) {
-    A v;
-    if (q == Q_MAX) {
-      if constexpr (F32ACC) {
-        v.hi = acc_max_f;
-        v.lo = 0.f;
-        for (int o = 16; o > 0; o >>= 1) v.hi = fmaxf(v.hi, __shfl_down_sync(0xffffffffu, v.hi, o));
-      } else {
-        v = acc_max;
-        for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_down_sync(0xffffffffu, v, o));
-      }
-    } else if (q < nq) {
-      v = acc[q];
+    for (int q = 0; q < NQ; ++q) {
+      if (q >= nq) continue;
+      A v = acc[q];
       for (int o = 16; o > 0; o >>= 1) acc_merge(v, shfl_down(v, o));
-    } else {
-      acc_zero(v);
+      if (lane == 0) red[warp][q] = v;
     }
-    if (lane == 0) red[warp][q] = v;
+  } else {
+    A v[16];
+#pragma unroll
+    for (int q = 0; q < 16; ++q) {
+      if (q < NQ && q != Q_MAX) v[q] = acc[q];
+      else acc_zero(v[q]);
+    }
+    A r = warp_reduce_scatter(v);
+    const int q = (lane >> 1) & 15;
+    // the root of the largest |.|^2 in the working precision (correctly
+    // rounded; a float64 root costs ~0.3 us and the float64 pipe)
+    A m;
+    if constexpr (F32ACC) {
+      float x = sqrtf((float)amax2);
+      for (int o = 16; o > 0; o >>= 1) x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, o));
+      m.hi = x;
+      m.lo = 0.f;
+    } else {
+      double x = amax2;
+      for (int o = 16; o > 0; o >>= 1) x = fmax(x, __shfl_xor_sync(0xffffffffu, x, o));
+      m = sqrt(x);
+    }
+    if (q == Q_MAX) r = m;
+    if ((lane & 1) == 0 && q < NQ) red[warp][q] = r;
   }
   __syncthreads();
   if (threadIdx.x < NQ) {
     const int q = threadIdx.x;
-    A v = red[0][q];
-    for (int w = 1; w < nw; ++w) {
-      if constexpr (std::is_same<A, double>::value) v = (q == Q_MAX) ? fmax(v, red[w][q]) : v + red[w][q];
-      else {
-        if (q == Q_MAX) df_max(v, red[w][q]);
+    A v;
+    acc_zero(v);
+    if (q < nq) {
+      v = red[0][q];
+      for (int w = 1; w < nw; ++w) {
+        if (q == Q_MAX) acc_max(v, red[w][q]);
         else acc_merge(v, red[w][q]);
       }
     }
@@ -401,90 +447,125 @@ static __device__ void block_partial(A (&acc)[NQ], M amax2, int nq, double* out)
   __syncthreads();
 }
 
-// Fold the partials of `tiles` consecutive CTAs (fixed order) into float64
-// out[0..NQ).  Called by one whole CTA.  Ends with a barrier.
+// Fold `rows` rows of partials, `stride` rows apart, in a fixed order; called by
+// one whole CTA.  Thread t takes quantity t mod 16 of the rows t / 16, t / 16 +
+// (threads / 16), ..., eight loads in flight; then lanes l and l + 16 and the
+// warps are joined.  Threads 0..NQ-1 return the sums (quantity = thread).
 template <typename A>
-static __device__ void fold_partials(const double* partials, int tiles, int nq, double* out) {
-  __shared__ A red[NTHREADS / 32][NQ];
+static __device__ A fold_rows(const double* partials, int rows, int stride, int nq) {
+  __shared__ A red[NTHREADS / 32][16];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int nw = blockDim.x >> 5;
-  A v[NQ];
+  const int nw = blockDim.x >> 5, slices = blockDim.x >> 4;
+  const int q = threadIdx.x & 15;
+  A x;
+  acc_zero(x);
+  if (q < nq) {
+    const A* pp = reinterpret_cast<const A*>(partials) + q;
+    const size_t rs = (size_t)stride * NQ;
+    for (int i0 = threadIdx.x >> 4; i0 < rows; i0 += 8 * slices) {
+      A w[8];
 #pragma unroll
-  for (int q = 0; q < NQ; ++q) acc_zero(v[q]);
-  const A* pp = reinterpret_cast<const A*>(partials);
-  for (int i = threadIdx.x; i < tiles; i += blockDim.x) {
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-      if (q >= nq && q != Q_MAX) continue;
-      A w;
-      if constexpr (std::is_same<A, double>::value) {
-        w = __ldcg(pp + (size_t)i * NQ + q);
-        v[q] = (q == Q_MAX) ? fmax(v[q], w) : v[q] + w;
-      } else {
-        const float2 f = __ldcg(reinterpret_cast<const float2*>(pp + (size_t)i * NQ + q));
-        w.hi = f.x;
-        w.lo = f.y;
-        if (q == Q_MAX) df_max(v[q], w);
-        else acc_merge(v[q], w);
-      }
-    }
-  }
-#pragma unroll
-  for (int q = 0; q < NQ; ++q) {
-    A x = v[q];
-    if (q < nq || q == Q_MAX) {
-      for (int o = 16; o > 0; o >>= 1) {
-        if constexpr (std::is_same<A, double>::value) {
-          const double w = __shfl_down_sync(0xffffffffu, x, o);
-          x = (q == Q_MAX) ? fmax(x, w) : x + w;
-        } else {
-          const DF w = shfl_down(x, o);
-          if (q == Q_MAX) df_max(x, w);
-          else acc_merge(x, w);
+      for (int u = 0; u < 8; ++u) {
+        const int i = i0 + u * slices;
+        acc_zero(w[u]);
+        if (i < rows) {
+          if constexpr (std::is_same<A, double>::value) {
+            w[u] = __ldcg(pp + i * rs);
+          } else {
+            const float2 f = __ldcg(reinterpret_cast<const float2*>(pp + i * rs));
+            w[u].hi = f.x;
+            w[u].lo = f.y;
+          }
         }
       }
-    } else {
-      acc_zero(x);
-    }
-    if (lane == 0) red[warp][q] = x;
-  }
-  __syncthreads();
-  if (threadIdx.x < NQ) {
-    const int q = threadIdx.x;
-    A x = red[0][q];
-    for (int w = 1; w < nw; ++w) {
-      if constexpr (std::is_same<A, double>::value) x = (q == Q_MAX) ? fmax(x, red[w][q]) : x + red[w][q];
-      else {
-        if (q == Q_MAX) df_max(x, red[w][q]);
-        else acc_merge(x, red[w][q]);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        if (q == Q_MAX) acc_max(x, w[u]);
+        else acc_merge(x, w[u]);
       }
     }
-    out[q] = acc_value(x);
+  }
+  {
+    const A w = shfl_xor(x, 16);
+    if (lane < 16) {
+      if (q == Q_MAX) acc_max(x, w);
+      else acc_merge(x, w);
+      red[warp][q] = x;
+    }
+  }
+  __syncthreads();
+  A v;
+  acc_zero(v);
+  if (threadIdx.x < NQ) {
+    const int k = threadIdx.x;
+    v = red[0][k];
+    for (int w = 1; w < nw; ++w) {
+      if (k == Q_MAX) acc_max(v, red[w][k]);
+      else acc_merge(v, red[w][k]);
+    }
+  }
+  return v;
+}
+
+// The sums of `tiles` consecutive CTAs' partials as float64 in res[0..NQ)
+// (shared memory) and out[0..NQ) (may be null).  Ends with a barrier.
+template <typename A>
+static __device__ void fold_partials(const double* partials, int tiles, int stride, int nq, double* out, double* res) {
+  const A v = fold_rows<A>(partials, tiles, stride, nq);
+  if (threadIdx.x < NQ) {
+    const double d = acc_value(v);
+    if (out) out[threadIdx.x] = d;
+    res[threadIdx.x] = d;
   }
   __syncthreads();
 }
 
-// Block partial, then the last CTA of the instance to finish (its own atomic
-// ticket) folds the instance's partials into results[inst][q].  Returns true in
-// that CTA.  One last CTA for the whole batch folded the instances one after
-// another, about 0.5 us for each sum: 64 us of the 82 us of a moments launch
-// over 128 instances.
+// Tickets of a launch of `blocks` CTAs over nb instances: one per instance and
+// one per group of FOLD_GROUP CTAs.
+constexpr int FOLD_GROUP = 16;
+static inline size_t fold_tickets(size_t blocks, size_t nb) { return 2 * nb + blocks / FOLD_GROUP + 1; }
+
+// Block partial; the last CTA of an instance to finish (atomic tickets) folds
+// the instance's partials into results[inst][q] and returns them (in shared
+// memory); the others return null.  One last CTA for the whole batch folded the
+// instances one after another, about 0.5 us for each sum: 64 us of the 82 us of
+// a moments launch over 128 instances.  Instances of more than FOLD_GROUP CTAs
+// are folded in two steps, each group by its own last CTA: one CTA of 64
+// threads took 10 us over the rows of 900 CTAs.
 template <typename A, typename M>
-static __device__ bool reduce_partials(A (&acc)[NQ], M amax2, int nq, double* partials, double* results,
-                                       unsigned int* ticket, int tiles_per_inst) {
+static __device__ const double* reduce_partials(A (&acc)[NQ], M amax2, int nq, double* partials, double* results,
+                                                unsigned int* ticket, int tiles) {
   __shared__ int s_last;
-  const int inst = blockIdx.x / tiles_per_inst;
-  block_partial(acc, amax2, nq, partials + (size_t)blockIdx.x * NQ);
-  __threadfence();
-  if (threadIdx.x == 0) s_last = (atomicAdd(ticket + inst, 1u) == (unsigned)tiles_per_inst - 1u);
-  __syncthreads();
-  if (!s_last) return false;
-  __threadfence();
-  fold_partials<A>(partials + (size_t)inst * tiles_per_inst * NQ, tiles_per_inst, nq, results + (size_t)inst * NQ);
-  if (threadIdx.x == 0) ticket[inst] = 0u;
-  __threadfence();
-  __syncthreads();
-  return true;
+  __shared__ double s_res[NQ];
+  const int inst = blockIdx.x / tiles, tile = blockIdx.x - inst * tiles;
+  double* base = partials + (size_t)inst * tiles * NQ;
+  block_partial(acc, amax2, nq, base + (size_t)tile * NQ);
+  auto last_of = [&](unsigned int* t, int n) -> bool {
+    __threadfence();
+    if (threadIdx.x == 0) {
+      s_last = atomicAdd(t, 1u) == (unsigned)n - 1u;
+      if (s_last) *t = 0u;
+    }
+    __syncthreads();
+    const bool l = s_last != 0;
+    if (l) __threadfence();
+    return l;
+  };
+  int rows = tiles, stride = 1;
+  if (tiles > FOLD_GROUP) {
+    const int ngroups = (tiles + FOLD_GROUP - 1) / FOLD_GROUP, g = tile / FOLD_GROUP;
+    const int n = min(FOLD_GROUP, tiles - g * FOLD_GROUP);
+    double* grow = base + (size_t)g * FOLD_GROUP * NQ;
+    if (!last_of(ticket + gridDim.x / tiles + inst * ngroups + g, n)) return nullptr;
+    const A v = fold_rows<A>(grow, n, 1, nq);
+    if (threadIdx.x < NQ) reinterpret_cast<A*>(grow)[threadIdx.x] = v;
+    __syncthreads();
+    rows = ngroups;
+    stride = FOLD_GROUP;
+  }
+  if (!last_of(ticket + inst, rows)) return nullptr;
+  fold_partials<A>(base, rows, stride, nq, results + (size_t)inst * NQ, s_res);
+  return s_res;
 }
 
 // Grid-wide barrier for a cooperative (co-resident) launch: arrival counter
@@ -920,10 +1001,10 @@ __device__ __forceinline__ void make_ctx(EpiCtx<T, CPLX>& E, const PassData<T>& 
 }
 
 template <typename T>
-__device__ __forceinline__ void run_control(const PassData<T>& D) {
-  if (threadIdx.x == 0) {
-    if (D.control == 1) alg1_control<T>(D.ctl, D.results);
-    else if (D.control == 2) rn_control(D.rn, D.results);
+__device__ __forceinline__ void run_control(const PassData<T>& D, const double* r) {
+  if (threadIdx.x == 0 && r) {
+    if (D.control == 1) alg1_control<T>(D.ctl, r);
+    else if (D.control == 2) rn_control(D.rn, r);
   }
 }
 
@@ -1115,7 +1196,7 @@ __global__ void __launch_bounds__(NTHREADS) k_pass(PassGeom<T> G, PassData<T> D)
   T amax = T(0);
   pass_tile<T, CPLX, EPI, false>(G, D, blockIdx.x, smem_raw, s_off, s_rc, acc, amax);
   if (EPI == EPI_ACC || EPI == EPI_HESS || D.nq == 0) return;
-  if (reduce_partials(acc, amax, D.nq, D.partials, D.results, D.ticket, G.tiles)) run_control<T>(D);
+  run_control<T>(D, reduce_partials(acc, amax, D.nq, D.partials, D.results, D.ticket, G.tiles));
 }
 
 // One launch runs a whole Algorithm 1 run (until the control block says done).
@@ -1203,7 +1284,7 @@ __global__ void __launch_bounds__(NTHREADS) k_alg1_persist(PersistArgs<T> P) {
       }
       stamp(loop, 1 + (a < 1 ? a : 1));
     }
-    fold_partials<A>(P.D.partials, P.blocks[P.dim - 1], NQ, s_res);
+    fold_partials<A>(P.D.partials, P.blocks[P.dim - 1], 1, NQ, nullptr, s_res);
     if (threadIdx.x == 0) alg1_control<T>(&s_ctl, s_res);
     __syncthreads();
     stamp(loop, 3);
@@ -1215,8 +1296,9 @@ __global__ void __launch_bounds__(NTHREADS) k_alg1_persist(PersistArgs<T> P) {
 // H_lin of §2.1 per axis (3/5/7-point, zero Dirichlet values outside) with the
 // central-difference rotation term, then the same epilogue as the spectral pass.
 // Float64 is bound by the float64 pipe (2 operations a clock and SM): the
-// diagonal is one coefficient per point, V + sum 1/h^2, and each axis adds one
-// addition and one multiply-add.
+// diagonal is one coefficient per point, V + sum 1/h^2, each axis adds one
+// addition and one multiply-add, and the CTAs are few (two per SM) because a
+// warp's reduction costs as much as two of its points.
 template <typename T, bool CPLX, int EPI>
 __global__ void __launch_bounds__(NTHREADS) k_fd(FDGeom G, const T* __restrict__ rx, const T* __restrict__ ry,
                                                 PassData<T> D) {
@@ -1300,7 +1382,7 @@ __global__ void __launch_bounds__(NTHREADS) k_fd(FDGeom G, const T* __restrict__
     epilogue_point<T, CPLX, EPI, 2>(E, base + li, x, lin, acc, amax);
   }
   if (EPI == EPI_HESS || D.nq == 0) return;
-  if (reduce_partials(acc, amax, D.nq, D.partials, D.results, D.ticket, G.tiles)) run_control<T>(D);
+  run_control<T>(D, reduce_partials(acc, amax, D.nq, D.partials, D.results, D.ticket, G.tiles));
 }
 
 // ----------------------------------------------------------------- elementwise kernels
@@ -1403,8 +1485,8 @@ __global__ void __launch_bounds__(NTHREADS) k_moments(const void* xv, const void
       }
     }
   }
-  if (reduce_partials(acc, T(0), 3, partials, results, ticket, tiles) && threadIdx.x == 0)
-    moment_coef(mc, inst, results + (size_t)inst * NQ);
+  const double* r = reduce_partials(acc, T(0), 3, partials, results, ticket, tiles);
+  if (r && threadIdx.x == 0) moment_coef(mc, inst, r);
 }
 
 // s a and s a + c with one rounding per operation whatever the compiler would

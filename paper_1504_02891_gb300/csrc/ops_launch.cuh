@@ -221,7 +221,8 @@ gpe_status GridDev<T>::create(const GridHost& g) {
       fd.ih2c[a] = a < g.dim ? 0.5 / g.h[a] : 0.0;
     }
     fd.omega = g.omega;
-    fd.tiles = (int)std::max<long long>(1, std::min<long long>((g.M + NTHREADS - 1) / NTHREADS, 1024));
+    fd.tiles = (int)std::max<long long>(
+        1, std::min<long long>((g.M + NTHREADS - 1) / NTHREADS, sizeof(T) == 8 ? std::max(16, 304 / g.nbatch) : 1024));
     fd_blocks = fd.tiles * g.nbatch;
     max_blocks = std::max(max_blocks, fd_blocks);
   }
@@ -462,6 +463,9 @@ gpe_status launch_axis_s(const GridHost& g, const GridDev<T>& d, int axis, const
 template <typename T, int EPI>
 gpe_status launch_axis_x(const GridHost& g, const GridDev<T>& d, const PassData<T>& D, cudaStream_t st);
 
+// Whether the 2D line kernels take the grid's shape (lines2d.cuh).
+template <typename T> bool lines2d_takes(const GridHost& g);
+
 // Epilogues the x line kernel runs: the float32 solver never runs the model
 // objective W, the float64 one never its difference form.  Float32 gradients
 // keep the general passes: energies of float32 states (and of steps made from
@@ -472,6 +476,14 @@ template <typename T> constexpr bool axis_x_takes(int epi) {
          (epi == EPI_GRAD && sizeof(T) == 8);
 }
 
+// Whether apply_op(EPI_WS, step_first) forms the difference-form step itself:
+// the first pass has to be a line kernel.
+template <typename T> bool shifted_step_ok(const GridHost& g) {
+  if (g.disc == GPE_FD) return false;
+  if (g.disc == GPE_FOURIER && g.dim == 2 && lines2d_takes<T>(g)) return true;
+  return axis_x_takes<T>(EPI_WS) && line_axis_ok(g, g.dim - 1);
+}
+
 // The axes from the last to x, each by its line kernel or, where that does not
 // take the line length, by the general axis pass; x has the epilogue.
 template <typename T>
@@ -479,7 +491,7 @@ gpe_status apply_axes(const GridHost& g, const GridDev<T>& d, const PassData<T>&
                       cudaStream_t st) {
   for (int a = g.dim - 1; a >= 0; --a) {
     PassData<T> Da = D;
-    Da.step_on_load = (step_first && a == g.dim - 1) ? 1 : 0;
+    Da.step_on_load = (step_first && a == g.dim - 1) ? (epi == EPI_WS ? 2 : 1) : 0;
     Da.acc_in = a < g.dim - 1 ? acc : nullptr;
     gpe_status s = GPE_OK;
     if (a > 0) {
@@ -626,6 +638,7 @@ gpe_status launch_alg1_persist(const GridHost& g, const GridDev<T>& d, const Pas
                                         const void*, void*, void*, void*, const double*, cudaStream_t);            \
   template gpe_status prolong_normalised<T>(const GridHost&, const GridHost&, const GridDev<T>&, const GridDev<T>&, \
                                             const void*, void*, void*, void*, double, Scratch&, cudaStream_t);     \
+  template bool shifted_step_ok<T>(const GridHost&);                                                                \
   template gpe_status apply_op<T>(const GridHost&, const GridDev<T>&, PassData<T>, int, void*, bool, cudaStream_t); \
   template gpe_status persist_config<T>(const GridHost&, const GridDev<T>&, int, int*, size_t*);                      \
   template gpe_status launch_alg1_persist<T>(const GridHost&, const GridDev<T>&, const PassData<T>&, void*,         \

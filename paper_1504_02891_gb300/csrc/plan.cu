@@ -235,8 +235,9 @@ gpe_status Scratch::create(size_t blocks, int nb) {
   GPE_CUDA(cudaMalloc(&partials, sizeof(double) * NQ * blocks));
   GPE_CUDA(cudaMalloc(&results, sizeof(double) * NQ * nb));
   GPE_CUDA(cudaMalloc(&coef, sizeof(double) * 4 * nb));
-  GPE_CUDA(cudaMalloc(&ticket, sizeof(unsigned int) * nb));
-  GPE_CUDA(cudaMemset(ticket, 0, sizeof(unsigned int) * nb));
+  const size_t tb = sizeof(unsigned int) * fold_tickets(blocks, nb);
+  GPE_CUDA(cudaMalloc(&ticket, tb));
+  GPE_CUDA(cudaMemset(ticket, 0, tb));
   GPE_CUDA(cudaMemset(results, 0, sizeof(double) * NQ * nb));
   GPE_CUDA(cudaMallocHost(&h_results, sizeof(double) * ((size_t)NQ * nb + 1)));
   h_results[(size_t)NQ * nb] = 0.0;

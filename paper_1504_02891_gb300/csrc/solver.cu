@@ -264,8 +264,9 @@ static gpe_status queue_iters(Level<T>& L, int objective, int n, cudaStream_t st
   const long long n_all = L.M * L.g.nbatch;   // elements (complex or real)
   for (int i = 0; i < n; ++i) {
     gpe_status s;
-    if (objective == 2) {
-      // difference form: the step needs X^k, so it runs as its own kernel
+    if (objective == 2 && !shifted_step_ok<T>(L.g)) {
+      // difference form on grids whose first pass does not form its step (which
+      // needs X^k): a kernel of its own
       s = launch_step<T>(D.xs, D.gs, D.ctl, n_all, L.g.is_complex, st, L.xk);
       if (s != GPE_OK) return s;
       s = apply_op<T>(L.g, L.d, D, epi, L.acc, false, st);
