@@ -159,9 +159,9 @@ typedef struct {
   int use_graphs;     /* capture the queued iterations in CUDA graphs           [1] */
   int persistent;     /* spectral grids: run each Algorithm 1 run as one
                          cooperative persistent launch (grid barriers with
-                         bounded waits; GPE_ETIMEOUT if one expires); 3D grids
-                         with 32..1024-point transforms on every axis (sine:
-                         real fields) queue their line kernels instead          [1] */
+                         bounded waits; GPE_ETIMEOUT if one expires); float64
+                         3D grids with 32..1024-point transforms on every axis
+                         (sine: real fields) queue their line kernels instead  [1] */
   int cluster;        /* float32 Algorithm 1 on 2D Fourier grids: one thread-block
                          cluster holds the whole state in distributed shared
                          memory (grids up to 256^2 complex)                      [1] */

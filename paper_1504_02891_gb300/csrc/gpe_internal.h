@@ -150,6 +150,14 @@ gpe_status launch_alg1_persist(const GridHost& g, const GridDev<T>& d, const Pas
                                unsigned int* bar, int* err, int max_loops, int epi, int grid, size_t smem,
                                cudaStream_t st);
 
+// The persistent float32 Algorithm 1 launch with line transforms
+// (persist_lines.cuh): F or the difference form WS; *launched is false on grids
+// it does not take.
+bool alg1_lines_ok(const GridHost& g);
+gpe_status launch_alg1_lines(const GridHost& g, const GridDev<float>& d, const PassData<float>& D, void* acc,
+                             unsigned int* bar, int* err, int max_loops, int epi, size_t cap_blocks, bool* launched,
+                             cudaStream_t st);
+
 // GPE_PERSIST_TRACE=1: phase timestamps of persistent launches (debug aid).
 unsigned long long* persist_debug_buffer(int* n);
 void persist_debug_report(cudaStream_t st, long long M, int f64);

@@ -859,6 +859,13 @@ struct EpiCtx {
   T nl, shift, lin_scale, th_c, delta, thk;
 };
 
+// One point of the objective passes (F, W, WS) with the current point's values
+// xc, gc at hand; base and gk are constant during a launch (read with COH).
+template <typename T, bool CPLX, int EPI, int COH = 2, typename A>
+__device__ __forceinline__ void epilogue_values(const EpiCtx<T, CPLX>& E, long long gi, typename VT<T, CPLX>::V x,
+                                                typename VT<T, CPLX>::V lin, typename VT<T, CPLX>::V xc,
+                                                typename VT<T, CPLX>::V gc, A (&acc)[NQ], T& amax);
+
 template <typename T, bool CPLX, int EPI, int COH = 0, typename A>
 __device__ __forceinline__ void epilogue_point(const EpiCtx<T, CPLX>& E, long long gi,
                                                typename VT<T, CPLX>::V x,
@@ -876,7 +883,35 @@ __device__ __forceinline__ void epilogue_point(const EpiCtx<T, CPLX>& E, long lo
     const T R = tre(p, x);
     // gathered by x and p: 12 operations a complex point instead of 18 (float64 issues 2 a clock)
     E.out[gi] = lin + (E.nl * p2 + E.shift) * x + (T(2) * E.nl * R) * p;
-  } else if (EPI == EPI_F || EPI == EPI_W) {
+  } else if (EPI == EPI_F || EPI == EPI_W || EPI == EPI_WS) {
+    const V xc = E.xc ? ldv<COH>(E.xc + gi) : vzero<V>();
+    const V gc = E.gc ? ldv<COH>(E.gc + gi) : vzero<V>();
+    epilogue_values<T, CPLX, EPI, COH>(E, gi, x, lin, xc, gc, acc, amax);
+  } else if (EPI == EPI_RATIO) {
+    const V d = x;
+    const V xk = ldv<COH>(E.base + gi);
+    const V gk = ldv<COH>(E.gk + gi);
+    const T x2 = tre(xk, xk);
+    const V ax = gk - (T(4) * E.nl * x2) * xk;
+    const V z = xk + d;
+    const T R = tre(xk, d), d2 = tre(d, d);
+    acc_add(acc[R_AXD], tre(ax, d));
+    acc_add(acc[R_DAD], T(2) * tre(d, lin));
+    acc_add(acc[R_QD], (T(2) * R + d2) * (tre(z, z) + x2));
+    acc_add(acc[R_X2D2], x2 * d2);
+    acc_add(acc[R_R2], R * R);
+    acc_add(acc[R_DD], d2);
+    acc_add(acc[R_GD], tre(gk, d));
+    amax = fmax(amax, d2);
+  }
+}
+
+template <typename T, bool CPLX, int EPI, int COH, typename A>
+__device__ __forceinline__ void epilogue_values(const EpiCtx<T, CPLX>& E, long long gi, typename VT<T, CPLX>::V x,
+                                                typename VT<T, CPLX>::V lin, typename VT<T, CPLX>::V xc,
+                                                typename VT<T, CPLX>::V gc, A (&acc)[NQ], T& amax) {
+  using V = typename VT<T, CPLX>::V;
+  if (EPI == EPI_F || EPI == EPI_W) {
     const V y = x;
     V g;
     if (EPI == EPI_F) {
@@ -900,8 +935,6 @@ __device__ __forceinline__ void epilogue_point(const EpiCtx<T, CPLX>& E, long lo
     const V q = g - E.th_c * y;
     acc_add(acc[Q_Q], tre(q, q));
     acc_add(acc[Q_QY], tre(q, y));
-    const V xc = E.xc ? ldv<COH>(E.xc + gi) : vzero<V>();
-    const V gc = E.gc ? ldv<COH>(E.gc + gi) : vzero<V>();
     const V s = y - xc;
     const V v = (g - gc) - E.th_c * s;
     const T s2 = tre(s, s);
@@ -937,9 +970,7 @@ __device__ __forceinline__ void epilogue_point(const EpiCtx<T, CPLX>& E, long lo
     const V q = gh - E.th_c * X;
     acc_add(acc[Q_Q], tre(q, q));
     acc_add(acc[Q_QY], tre(q, X));
-    const V yc = E.xc ? ldv<COH>(E.xc + gi) : vzero<V>();
-    const V gc = E.gc ? ldv<COH>(E.gc + gi) : vzero<V>();
-    const V s = y - yc;
+    const V s = y - xc;
     const V v = (gh - gc) - E.th_c * s;
     const T s2 = tre(s, s);
     acc_add(acc[Q_SS], s2);
@@ -949,22 +980,6 @@ __device__ __forceinline__ void epilogue_point(const EpiCtx<T, CPLX>& E, long lo
     acc_add(acc[Q_SY], tre(s, X));
     acc_add(acc[Q_DF], tre(s, q) - T(0.5) * tre(s, v));   // the model is quadratic: trapezoid exact
     amax = fmax(amax, s2);
-  } else if (EPI == EPI_RATIO) {
-    const V d = x;
-    const V xk = ldv<COH>(E.base + gi);
-    const V gk = ldv<COH>(E.gk + gi);
-    const T x2 = tre(xk, xk);
-    const V ax = gk - (T(4) * E.nl * x2) * xk;
-    const V z = xk + d;
-    const T R = tre(xk, d), d2 = tre(d, d);
-    acc_add(acc[R_AXD], tre(ax, d));
-    acc_add(acc[R_DAD], T(2) * tre(d, lin));
-    acc_add(acc[R_QD], (T(2) * R + d2) * (tre(z, z) + x2));
-    acc_add(acc[R_X2D2], x2 * d2);
-    acc_add(acc[R_R2], R * R);
-    acc_add(acc[R_DD], d2);
-    acc_add(acc[R_GD], tre(gk, d));
-    amax = fmax(amax, d2);
   }
 }
 

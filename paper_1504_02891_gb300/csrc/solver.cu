@@ -355,12 +355,27 @@ static gpe_status alg1_run(Level<T>& L, int objective, int first_slot, int max_i
   long long launched = 0;
   s = read_ctl<T>(L, st);
   if (s != GPE_OK) return s;
-  // 3D grids that the line kernels take run faster as queued chunks of them
-  // than as one persistent launch of general pass tiles (64^3 sine float32: 16
-  // against 60 us an iteration)
+  // float32 on square and cubic grids: one persistent launch of line transforms
+  if constexpr (std::is_same<T, float>::value) {
+    if (!L.h_ctl->done && P.persistent && objective != 1 && !prof_enabled()) {
+      bool ran = false;
+      s = launch_alg1_lines(L.g, L.d, L.solver_data(objective), L.acc, L.bar, L.err, (int)max_launch,
+                            objective_epi(objective), L.sc.cap_blocks, &ran, st);
+      if (s != GPE_OK) return s;
+      if (ran) {
+        GPE_CUDA(cudaMemcpyAsync(L.h_err, L.err, sizeof(int), cudaMemcpyDeviceToHost, st));
+        s = read_ctl<T>(L, st);
+        if (s != GPE_OK) return s;
+        if (*L.h_err) return fail(GPE_ETIMEOUT, "a grid barrier wait of the persistent Algorithm 1 launch expired");
+        launched = max_launch;
+      }
+    }
+  }
+  // float64 3D grids that the line kernels take run faster as queued chunks of
+  // them than as one persistent launch of general pass tiles
   bool queued = L.g.dim == 3;
   for (int a = 0; a < L.g.dim; ++a) queued = queued && line_axis_ok(L.g, a);
-  if (!L.h_ctl->done && P.persistent && !queued && objective < 2 && !prof_enabled()) {
+  if (!L.h_ctl->done && launched < max_launch && P.persistent && !queued && objective < 2 && !prof_enabled()) {
     if (L.p_grid[objective] < 0) {
       s = persist_config<T>(L.g, L.d, objective == 1 ? EPI_W : EPI_F, &L.p_grid[objective], &L.p_smem[objective]);
       if (s != GPE_OK) return s;
@@ -646,6 +661,9 @@ static gpe_status fg_run_cluster(Level<float>& L, const SolveParams& P, bool sto
   *used = false;
   const GridHost& g = L.g;
   if (!P.cluster || g.disc != GPE_FOURIER || g.dim != 2 || prof_enabled()) return GPE_OK;
+  // 256^2 complex: the line transforms on 64 CTAs and a grid barrier take 15.7
+  // us a trial, 16 CTAs with the state in shared memory 20.6
+  if (P.persistent && g.is_complex && g.M >= 65536 && alg1_lines_ok(g)) return GPE_OK;
   int cs, lch, P0, P1;
   size_t smem;
   unsigned int vb, vp;
