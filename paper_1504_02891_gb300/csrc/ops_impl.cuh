@@ -1200,6 +1200,8 @@ __device__ __forceinline__ void pass_tile(const PassGeom<T>& G, const PassData<T
 
 template <typename T, bool CPLX, int EPI>
 __global__ void __launch_bounds__(NTHREADS) k_pass(PassGeom<T> G, PassData<T> D) {
+  pdl_next();
+  pdl_wait();
   if (D.ctl && D.ctl->done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ long long s_off[MAXLB];
@@ -1318,6 +1320,8 @@ template <typename T, bool CPLX, int EPI>
 __global__ void __launch_bounds__(NTHREADS) k_fd(FDGeom G, const T* __restrict__ rx, const T* __restrict__ ry,
                                                 PassData<T> D) {
   using V = typename VT<T, CPLX>::V;
+  pdl_next();
+  pdl_wait();
   if (D.ctl && D.ctl->done) return;
   const int inst = blockIdx.x / G.tiles;
   const int tb = blockIdx.x - inst * G.tiles;

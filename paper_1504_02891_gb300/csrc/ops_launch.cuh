@@ -250,6 +250,12 @@ void GridDev<T>::destroy() {
   fsync = nullptr;
 }
 
+// Float32 passes of the entry points (no solver slots) with the length known,
+// transforms of 32 to 1024 points (pass_f32.cuh).
+template <bool CPLX, int EPI>
+gpe_status launch_pass_s(const PassGeom<float>& G, int blocks, const PassData<float>& D, size_t smem,
+                         cudaStream_t st);
+
 template <typename T, bool CPLX, int EPI>
 static gpe_status launch_pass_t(const PassGeom<T>& G, int blocks, const PassData<T>& D, cudaStream_t st) {
   using C = typename C2t<T>::type;
@@ -257,10 +263,12 @@ static gpe_status launch_pass_t(const PassGeom<T>& G, int blocks, const PassData
   const int nst = 1 + ((D.xsub || D.step_on_load) ? 1 : 0) + (D.acc_in ? 1 : 0);
   const size_t smem = (size_t)G.F * sizeof(C) + 2 * (size_t)G.LC * G.P * sizeof(C) +
                       (size_t)nst * G.LB * G.len * vsz + (EPI != EPI_ACC ? (size_t)G.LB * G.len * sizeof(T) : 0);
+  if constexpr (std::is_same<T, float>::value && (EPI == EPI_ACC || EPI == EPI_GRAD)) {
+    if (!D.ctl && !D.xsub && G.logF >= 5 && G.logF <= 10) return launch_pass_s<CPLX, EPI>(G, blocks, D, smem, st);
+  }
   GPE_CUDA(raise_smem((const void*)k_pass<T, CPLX, EPI>, smem));
   ProfScope ps(kernel_name("pass", sizeof(T) == 8, CPLX, EPI, G.M * (blocks / G.tiles)), st);
-  k_pass<T, CPLX, EPI><<<blocks, G.nthreads, smem, st>>>(G, D);
-  GPE_CUDA(cudaGetLastError());
+  GPE_CUDA(launch_pdl(k_pass<T, CPLX, EPI>, blocks, G.nthreads, smem, st, G, D));
   return GPE_OK;
 }
 
@@ -291,8 +299,8 @@ gpe_status launch_fd(const GridDev<T>& d, const PassData<T>& D, int cplx, int ep
   ProfScope ps(kernel_name("fd", sizeof(T) == 8, cplx, epi, d.fd.M * (d.fd_blocks / d.fd.tiles)), st);
 #define GPE_FD_CASE(E)                                                                                   \
   case E:                                                                                                \
-    if (cplx) k_fd<T, true, E><<<d.fd_blocks, NTHREADS, 0, st>>>(d.fd, rx, ry, D);                        \
-    else k_fd<T, false, E><<<d.fd_blocks, NTHREADS, 0, st>>>(d.fd, rx, ry, D);                            \
+    if (cplx) GPE_CUDA(launch_pdl(k_fd<T, true, E>, d.fd_blocks, NTHREADS, 0, st, d.fd, rx, ry, D));      \
+    else GPE_CUDA(launch_pdl(k_fd<T, false, E>, d.fd_blocks, NTHREADS, 0, st, d.fd, rx, ry, D));          \
     break;
   switch (epi) {
     GPE_FD_CASE(EPI_GRAD)
