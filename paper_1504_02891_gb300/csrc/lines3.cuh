@@ -23,8 +23,10 @@
 // float32 issue counts (46% of the cycles of the float32 strided kernel, 23% of
 // the warps resident); on 64^3 a kernel is a chain of a few latencies.
 // Measured against the general passes (a shared-memory tile per axis): 127^3
-// sine gradient float64 1039 -> 245 us, Hessian-vector float32 117 -> 59 us, 3D
-// rotating 32 x 128 x 128 float32 47 -> 20 us, 512 points float64 35 -> 24 us.
+// sine gradient float64 1039 -> 208 us, Hessian-vector float32 117 -> 46 us
+// (245 and 59 before the register budget below, the two-level folds and the
+// programmatic launches), energy of 512 points float64 52 -> 26.5 us (with the
+// pinned sums).
 #pragma once
 #include "lines2d.cuh"
 
@@ -40,6 +42,14 @@ template <typename T> __host__ __device__ constexpr int axs_cw(int lf) {
   return sizeof(T) == 4 ? (lf <= 9 ? 8 : 4) : (lf <= 6 ? 8 : (lf <= 9 ? 4 : 2));
 }
 template <typename T> __host__ __device__ constexpr int axs_threads(int lf) { return axs_cw<T>(lf) * (1 << lf) / 8; }
+// Resident CTAs the strided kernel's registers are sized for: 24 warps per SM in
+// float32 (85 registers) and 16 in float64 (128), where the compiler's own
+// choice (92 and 168) left room for 16 and 12 (127^3: Hessian-vector float32
+// 48.5 -> 45.6 us, gradient float64 217 -> 208).
+template <typename T> __host__ __device__ constexpr int axs_minb(int lf) {
+  const int warps = sizeof(T) == 4 ? 24 : 16, w = axs_threads<T>(lf) / 32;
+  return axs_threads<T>(lf) >= (sizeof(T) == 4 ? 512 : 256) ? 1 : warps / w;
+}
 // Threads of the x-kernel's CTA: 128 in float32, 64 in float64 (which lowers
 // the tail of small grids), or one line's.
 template <typename T> __host__ __device__ constexpr int axx_threads(int lf) {
@@ -68,7 +78,7 @@ __device__ __forceinline__ void mirror_odd(C (&v)[8], const Ex& ex, int& par, in
 
 // Strided axis: out = (acc_in or 0) + T_a X over the tiles of all planes.
 template <typename T, int KIND, int LF>
-__global__ void __launch_bounds__(axs_threads<T>(LF)) k_axis_s(PassGeom<T> G, PassData<T> D, int width, int tiles) {
+__global__ void __launch_bounds__(axs_threads<T>(LF), axs_minb<T>(LF)) k_axis_s(PassGeom<T> G, PassData<T> D, int width, int tiles) {
   using FFT = LineFFT<T, LF>;
   using C = typename FFT::C;
   using X = typename FFT::X;
@@ -381,7 +391,9 @@ static gpe_status launch_axis_x_t(const GridDev<T>& d, const PassData<T>& D, int
   const long long rows = G.M / G.len;
   const long long lines = KIND == LK_CPLX ? rows : (rows + 1) / 2;
   const int groups = (int)((lines + NL - 1) / NL);
-  // one resident wave (each CTA pays a reduction of its sums), within the reduction scratch
+  // one resident wave (each CTA pays its tables and a reduction of its sums; a
+  // CTA per group took 47.8 us for the 127^3 Hessian-vector product, this 45.6),
+  // within the reduction scratch
   long long cap = std::min<long long>((long long)sh.occ * num_sms(), d.max_blocks);
   const int tiles = (int)std::max<long long>(1, std::min<long long>(groups, std::max<long long>(cap / nbatch, 1)));
   if ((long long)tiles * nbatch > d.max_blocks) return fail(GPE_EINVAL, "reduction scratch too small");

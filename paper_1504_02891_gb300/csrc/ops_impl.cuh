@@ -389,10 +389,10 @@ __device__ __forceinline__ void acc_max(double& a, double b) { a = fmax(a, b); }
 
 // Reduce the per-thread sums acc[0..nq) over the block and write this CTA's
 // partials to out[0..NQ); the other slots are 0.  Slot Q_MAX, the largest |.|
-// (amax2: its square), is reduced when all NQ slots are asked for.  Ends with
-// a barrier.
+// (amax2: its square), is reduced when all NQ slots are asked for.  Threads
+// 0..NQ-1 return the sums (quantity = thread).  Ends with a barrier.
 template <typename A, typename M>
-static __device__ void block_partial(A (&acc)[NQ], M amax2, int nq, double* out) {
+static __device__ A block_partial(A (&acc)[NQ], M amax2, int nq, double* out) {
   constexpr bool F32ACC = !std::is_same<A, double>::value;
   __shared__ A red[NTHREADS / 32][16];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -431,10 +431,10 @@ static __device__ void block_partial(A (&acc)[NQ], M amax2, int nq, double* out)
     if ((lane & 1) == 0 && q < NQ) red[warp][q] = r;
   }
   __syncthreads();
+  A v;
+  acc_zero(v);
   if (threadIdx.x < NQ) {
     const int q = threadIdx.x;
-    A v;
-    acc_zero(v);
     if (q < nq) {
       v = red[0][q];
       for (int w = 1; w < nw; ++w) {
@@ -445,6 +445,7 @@ static __device__ void block_partial(A (&acc)[NQ], M amax2, int nq, double* out)
     reinterpret_cast<A*>(out)[q] = v;
   }
   __syncthreads();
+  return v;
 }
 
 // Fold `rows` rows of partials, `stride` rows apart, in a fixed order; called by
@@ -539,7 +540,12 @@ static __device__ const double* reduce_partials(A (&acc)[NQ], M amax2, int nq, d
   __shared__ double s_res[NQ];
   const int inst = blockIdx.x / tiles, tile = blockIdx.x - inst * tiles;
   double* base = partials + (size_t)inst * tiles * NQ;
-  block_partial(acc, amax2, nq, base + (size_t)tile * NQ);
+  const A own = block_partial(acc, amax2, nq, base + (size_t)tile * NQ);
+  if (tiles == 1) {   // nobody to wait for
+    if (threadIdx.x < NQ) results[(size_t)inst * NQ + threadIdx.x] = s_res[threadIdx.x] = acc_value(own);
+    __syncthreads();
+    return s_res;
+  }
   auto last_of = [&](unsigned int* t, int n) -> bool {
     __threadfence();
     if (threadIdx.x == 0) {
