@@ -546,16 +546,18 @@ static __device__ const double* reduce_partials(A (&acc)[NQ], M amax2, int nq, d
     __syncthreads();
     return s_res;
   }
+  // called after a barrier: thread 0's fences cover the CTA's writes and reads
   auto last_of = [&](unsigned int* t, int n) -> bool {
-    __threadfence();
     if (threadIdx.x == 0) {
+      __threadfence();
       s_last = atomicAdd(t, 1u) == (unsigned)n - 1u;
-      if (s_last) *t = 0u;
+      if (s_last) {
+        *t = 0u;
+        __threadfence();
+      }
     }
     __syncthreads();
-    const bool l = s_last != 0;
-    if (l) __threadfence();
-    return l;
+    return s_last != 0;
   };
   int rows = tiles, stride = 1;
   if (tiles > FOLD_GROUP) {
@@ -867,10 +869,15 @@ struct EpiCtx {
 
 // One point of the objective passes (F, W, WS) with the current point's values
 // xc, gc at hand; base and gk are constant during a launch (read with COH).
+// diff: there is a current point.  A run's first evaluation has none and its
+// control reads no difference sum (slots Q_SS.. and Q_MAX); in float64 they are
+// half of the 36 operations a point, of which an SM sub-partition issues one
+// warp's in 64 clocks: they were 37 of the 80 thousand cycles of the 256^2 real
+// x-kernel (49 -> 44.5 us without the differences).
 template <typename T, bool CPLX, int EPI, int COH = 2, typename A>
 __device__ __forceinline__ void epilogue_values(const EpiCtx<T, CPLX>& E, long long gi, typename VT<T, CPLX>::V x,
                                                 typename VT<T, CPLX>::V lin, typename VT<T, CPLX>::V xc,
-                                                typename VT<T, CPLX>::V gc, A (&acc)[NQ], T& amax);
+                                                typename VT<T, CPLX>::V gc, A (&acc)[NQ], T& amax, bool diff = true);
 
 template <typename T, bool CPLX, int EPI, int COH = 0, typename A>
 __device__ __forceinline__ void epilogue_point(const EpiCtx<T, CPLX>& E, long long gi,
@@ -892,7 +899,7 @@ __device__ __forceinline__ void epilogue_point(const EpiCtx<T, CPLX>& E, long lo
   } else if (EPI == EPI_F || EPI == EPI_W || EPI == EPI_WS) {
     const V xc = E.xc ? ldv<COH>(E.xc + gi) : vzero<V>();
     const V gc = E.gc ? ldv<COH>(E.gc + gi) : vzero<V>();
-    epilogue_values<T, CPLX, EPI, COH>(E, gi, x, lin, xc, gc, acc, amax);
+    epilogue_values<T, CPLX, EPI, COH>(E, gi, x, lin, xc, gc, acc, amax, sizeof(T) == 4 || E.xc != nullptr);
   } else if (EPI == EPI_RATIO) {
     const V d = x;
     const V xk = ldv<COH>(E.base + gi);
@@ -915,7 +922,7 @@ __device__ __forceinline__ void epilogue_point(const EpiCtx<T, CPLX>& E, long lo
 template <typename T, bool CPLX, int EPI, int COH, typename A>
 __device__ __forceinline__ void epilogue_values(const EpiCtx<T, CPLX>& E, long long gi, typename VT<T, CPLX>::V x,
                                                 typename VT<T, CPLX>::V lin, typename VT<T, CPLX>::V xc,
-                                                typename VT<T, CPLX>::V gc, A (&acc)[NQ], T& amax) {
+                                                typename VT<T, CPLX>::V gc, A (&acc)[NQ], T& amax, bool diff) {
   using V = typename VT<T, CPLX>::V;
   if (EPI == EPI_F || EPI == EPI_W) {
     const V y = x;
@@ -941,6 +948,7 @@ __device__ __forceinline__ void epilogue_values(const EpiCtx<T, CPLX>& E, long l
     const V q = g - E.th_c * y;
     acc_add(acc[Q_Q], tre(q, q));
     acc_add(acc[Q_QY], tre(q, y));
+    if (!diff) return;
     const V s = y - xc;
     const V v = (g - gc) - E.th_c * s;
     const T s2 = tre(s, s);
