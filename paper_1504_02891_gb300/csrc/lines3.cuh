@@ -17,11 +17,13 @@
 //
 // The odd half of a sine line is mirrored through the exchange buffer, so each
 // value is read from memory once.  The operands of the epilogue are fetched
-// (registers in float32, cp.async slots in float64) before the transforms.
+// (registers in float32, cp.async slots in float64) before the transforms, or
+// on large float64 grids after them (see launch_axis_x_t).
 //
 // What bounds them: on 128^3 grids the arrays stay in L2 and the integer and
-// float32 issue counts (46% of the cycles of the float32 strided kernel, 23% of
-// the warps resident); on 64^3 a kernel is a chain of a few latencies.
+// float32 issue counts (half of the cycles of the strided kernels, with 32% of
+// the warps resident in float32 and 23% in float64); on 64^3 a kernel is a
+// chain of a few latencies.
 // Measured against the general passes (a shared-memory tile per axis): 127^3
 // sine gradient float64 1039 -> 208 us, Hessian-vector float32 117 -> 46 us
 // (245 and 59 before the register budget below, the two-level folds and the
@@ -205,7 +207,8 @@ __global__ void __launch_bounds__(axs_threads<T>(LF), axs_minb<T>(LF)) k_axis_s(
 // of an instance takes the line groups tile, tile + tiles_per_inst, ...
 template <typename T, int KIND, int EPI, int LF>
 __global__ void __launch_bounds__(axx_threads<T>(LF), axx_minb<T>(LF)) k_axis_x(PassGeom<T> G, PassData<T> D,
-                                                                              int tiles_per_inst, int groups) {
+                                                                              int tiles_per_inst, int groups,
+                                                                              int slots) {
   using FFT = LineFFT<T, LF>;
   using C = typename FFT::C;
   using X = typename FFT::X;
@@ -219,8 +222,8 @@ __global__ void __launch_bounds__(axx_threads<T>(LF), axx_minb<T>(LF)) k_axis_x(
   extern __shared__ __align__(16) unsigned char smem_raw[];
   typename FFT::Tw* tws = reinterpret_cast<typename FFT::Tw*>(smem_raw);
   X* xb = reinterpret_cast<X*>(tws + F);         // [2][NL][P]
-  V* es = reinterpret_cast<V*>(xb + 2 * NL * FFT::P);   // float64: [2][NV][NT] input, accumulator
-  T* ev = reinterpret_cast<T*>(es + 2 * NV * NT);       // [NV][NT] potential
+  V* es = reinterpret_cast<V*>(xb + 2 * NL * FFT::P);   // float64: [NV][NT] input, with slots [2] (accumulator)
+  T* ev = reinterpret_cast<T*>(es + 2 * NV * NT);       // with slots: [NV][NT] potential
   __shared__ long long s_red[(NT + 31) / 32];
   load_table(tws, line_table<FFT>(G), F);
   const int tid = threadIdx.x;
@@ -305,7 +308,7 @@ __global__ void __launch_bounds__(axx_threads<T>(LF), axx_minb<T>(LF)) k_axis_x(
           vv[q] = Vp[at(q)];
         }
       } else {
-        if (has(q)) {
+        if (slots && has(q)) {
           if (accin) cp_async(es + (NV + q) * NT + tid, accin + ibase + at(q));
           cp_async(ev + q * NT + tid, Vp + at(q));
         }
@@ -330,27 +333,43 @@ __global__ void __launch_bounds__(axx_threads<T>(LF), axx_minb<T>(LF)) k_axis_x(
     if constexpr (KIND == LK_SINE) mirror_odd<T, LF>(v, ex, par, j);
     sym.c1c = (CPLX && G.rcoord && r0 < rows) ? G.c1 * G.rcoord[r0 % G.n1] : T(0);
     fft.apply(v, ex, par, sym);
-    if constexpr (!REGS) cp_async_wait_all();
-#pragma unroll
-    for (int q = 0; q < NV; ++q) {
-      if (!has(q)) continue;
-      V kin, x;
+    auto point = [&](int q, V x, V aq, T pv) {
+      V kin;
       if constexpr (CPLX) kin = v[q];
       else kin = q < NP ? v[q % NP].x : v[q % NP].y;
-      T pv;
-      if constexpr (REGS) {
-        x = xv[q];
-        kin = kin + av[q];
-        pv = vv[q];
-      } else {
-        x = es[q * NT + tid];
-        if (accin) kin = kin + es[(NV + q) * NT + tid];
-        pv = ev[q * NT + tid];
-      }
+      if (REGS || accin) kin = kin + aq;
       const V lin = kin + pv * x;
       // (read-only loads of the other vectors: plain ones would each wait for
       // the store before it)
       epilogue_point<T, CPLX, EPI, 2>(E, ibase + at(q), x, lin, acc, amax);
+    };
+    if constexpr (REGS) {
+#pragma unroll
+      for (int q = 0; q < NV; ++q)
+        if (has(q)) point(q, xv[q], av[q], vv[q]);
+    } else if (slots) {
+      cp_async_wait_all();
+#pragma unroll
+      for (int q = 0; q < NV; ++q)
+        if (has(q)) point(q, es[q * NT + tid], accin ? es[(NV + q) * NT + tid] : vzero<V>(), ev[q * NT + tid]);
+    } else {
+      constexpr int NE = NV < 8 ? NV : 8;   // values whose operands are in flight together
+#pragma unroll
+      for (int q0 = 0; q0 < NV; q0 += NE) {
+        V ac[NE];
+        T pc[NE];
+#pragma unroll
+        for (int u = 0; u < NE; ++u) {
+          ac[u] = vzero<V>();
+          pc[u] = T(0);
+          if (!has(q0 + u)) continue;
+          if (accin) ac[u] = ldv<2>(accin + ibase + at(q0 + u));
+          pc[u] = ldv<2>(Vp + at(q0 + u));
+        }
+#pragma unroll
+        for (int u = 0; u < NE; ++u)
+          if (has(q0 + u)) point(q0 + u, es[(q0 + u) * NT + tid], ac[u], pc[u]);
+      }
     }
   }
   if (EPI == EPI_HESS || D.nq == 0) return;
@@ -384,13 +403,25 @@ static gpe_status launch_axis_x_t(const GridDev<T>& d, const PassData<T>& D, int
   constexpr int NT = axx_threads<T>(LF), NL = NT / FFT::TPL;
   constexpr int NV = KIND == LK_REAL ? 16 : 8;
   const size_t vsz = sizeof(T) * (KIND == LK_CPLX ? 2 : 1);
-  const size_t smem = (size_t)FFT::F * sizeof(typename FFT::Tw) + 2 * (size_t)NL * FFT::P * sizeof(typename FFT::X) +
-                      (sizeof(T) == 8 ? (size_t)NV * NT * (2 * vsz + sizeof(T)) : 0);
-  static const KernelShape sh = kernel_shape((const void*)k_axis_x<T, KIND, EPI, LF>, NT, smem);
-  GPE_CUDA(sh.e);
+  const size_t base = (size_t)FFT::F * sizeof(typename FFT::Tw) + 2 * (size_t)NL * FFT::P * sizeof(typename FFT::X);
+  const size_t few = base + (sizeof(T) == 8 ? (size_t)NV * NT * vsz : 0);
+  const size_t all = base + (sizeof(T) == 8 ? (size_t)NV * NT * (2 * vsz + sizeof(T)) : 0);
+  static const KernelShape sf = kernel_shape((const void*)k_axis_x<T, KIND, EPI, LF>, NT, few);
+  static const KernelShape sa = kernel_shape((const void*)k_axis_x<T, KIND, EPI, LF>, NT, all);
+  GPE_CUDA(sf.e);
+  GPE_CUDA(sa.e);
   const long long rows = G.M / G.len;
   const long long lines = KIND == LK_CPLX ? rows : (rows + 1) / 2;
   const int groups = (int)((lines + NL - 1) / NL);
+  // float64: shared-memory slots for the epilogue's operands hide their latency
+  // behind the transforms, but cost resident CTAs.  With more than two and a half
+  // waves of groups the operands are loaded after the transforms instead (128^3
+  // real Fourier gradient 165 -> 147 us, 127^3 sine gradient 208.4 -> 206.5 and
+  // Hessian-vector 188.6 -> 186.2; at 2.2 waves, four 64^3 complex gradients,
+  // 151 against 153, at 1.6, three 64^3 sine gradients, 114 against 122)
+  const int slots = sizeof(T) == 8 && 2LL * groups * nbatch <= 5LL * sa.occ * num_sms();
+  const KernelShape& sh = slots ? sa : sf;
+  const size_t smem = slots ? all : few;
   // one resident wave (each CTA pays its tables and a reduction of its sums; a
   // CTA per group took 47.8 us for the 127^3 Hessian-vector product, this 45.6),
   // within the reduction scratch
@@ -398,7 +429,7 @@ static gpe_status launch_axis_x_t(const GridDev<T>& d, const PassData<T>& D, int
   const int tiles = (int)std::max<long long>(1, std::min<long long>(groups, std::max<long long>(cap / nbatch, 1)));
   if ((long long)tiles * nbatch > d.max_blocks) return fail(GPE_EINVAL, "reduction scratch too small");
   ProfScope ps(kernel_name("axis_x", sizeof(T) == 8, KIND == LK_CPLX, EPI, G.M * nbatch), st);
-  GPE_CUDA(launch_pdl(k_axis_x<T, KIND, EPI, LF>, nbatch * tiles, NT, smem, st, G, D, tiles, groups));
+  GPE_CUDA(launch_pdl(k_axis_x<T, KIND, EPI, LF>, nbatch * tiles, NT, smem, st, G, D, tiles, groups, slots));
   return GPE_OK;
 }
 

@@ -46,3 +46,26 @@ def test_operator_matches_oracle(n, disc, prec, tol, cplx):
         assert abs(E[b] - O.energy(g, x)) <= tol * abs(E[b])
         ref = O.apply_hlin(g, e) + g.beta * (np.abs(x) ** 2 * e + 2 * np.real(np.conj(x) * e) * x) + 0.25 * e
         assert np.max(np.abs(hv[b] - ref)) <= tol * np.max(np.abs(ref))
+
+
+# A batch of more than two waves of line groups per device: float64 x-kernels
+# then load the epilogue's operands after the transforms, and a CTA of the
+# float32 2D y-kernel takes several groups.  The arithmetic of a point does not
+# depend on the batch: the same bits as one instance alone.
+@pytest.mark.parametrize("n,disc,cplx,prec,nb", [
+    ((32, 32, 32), "fourier", False, G.F64, 97), ((32, 32, 32), "fourier", True, G.F64, 49),
+    ((16, 16, 16), "sine", False, G.F64, 401), ((64,), "fourier", True, G.F64, 2603),
+    ((512,), "fourier", False, G.F64, 1601), ((64, 128), "fourier", True, G.F32, 401),
+    ((128, 64), "fourier", False, G.F32, 801)])
+def test_large_batches_repeat_single_instances(n, disc, cplx, prec, nb):
+    d = len(n)
+    p = W.problem(d, n, (-8.0,) * d, (8.0, 7.0, 6.0)[:d], disc, beta=50.0, omega=0.5 if cplx and d > 1 else 0.0,
+                  is_complex=cplx, potential={"kind": "harmonic", "gamma": (1.0, 1.2, 1.5)[:d]})
+    psi = G.to_device(np.stack([W.random_field(p, seed=s % 7) * (1.0 + 0.01 * s) for s in range(nb)]), prec)
+    dd = G.to_device(np.stack([W.random_field(p, seed=20 + s % 5) for s in range(nb)]), prec)
+    with G.Plan(p, nbatch=nb, prec=prec) as plan:
+        out, hv = plan.grad(psi), plan.hessvec(psi, dd, 0.25)
+    with G.Plan(p, nbatch=1, prec=prec) as plan:
+        for b in (0, 1, nb // 2, nb - 1):
+            assert torch.equal(out[b], plan.grad(psi[b:b + 1].contiguous()).reshape(out[b].shape))
+            assert torch.equal(hv[b], plan.hessvec(psi[b:b + 1].contiguous(), dd[b:b + 1].contiguous(), 0.25).reshape(hv[b].shape))
