@@ -264,7 +264,7 @@ gpe_status gpe_solve_batch(const gpe_problem* problems, int n, void* const* psi,
  *     gives a distinct cluster size;
  * and records the fastest choices in a process-wide table keyed by grid (and
  * batch), which every later launch on those shapes uses (without an entry:
- * 4 waves, 4 KiB).  Launch shapes do not change computed values (reductions
+ * 4 waves, 1 for the float32 columns, 4 KiB).  Launch shapes do not change computed values (reductions
  * may differ by rounding order); the fused-or-two-kernel choice changes the
  * FFT factorisation, so operator values agree to rounding.  Other grids: nothing to tune, GPE_OK.  Allocates scratch
  * of two plan vectors and one solver level per grid; synchronises.  Not

@@ -13,7 +13,8 @@
 //   * float32 square 2D Fourier grids: the fused one-launch operator kernel
 //     (fused2d.cuh) or the two line kernels, whichever applies the operator
 //     faster for the grid and batch.
-// Launches with no table entry use the fixed rule (4 waves; 4 KiB; the fused
+// Launches with no table entry use the fixed rule (4 waves, the
+// float32 column kernel 1; 4 KiB; the fused
 // kernel for batches of >= 16 instances on grids up to 256^2).  The
 // choice never changes what is computed, only how the work is spread: the
 // operator values are identical, reductions may differ by rounding order.
@@ -51,7 +52,11 @@ void set_tuned_fused(int cplx, int n, int nbatch, int on) {
 int tuned_waves(int axis, int prec64, int cplx, int n0, int n1, int nbatch) {
   std::lock_guard<std::mutex> lk(g_mu);
   auto it = g_waves.find(std::make_tuple(prec64, cplx, n0, n1, nbatch));
-  if (it == g_waves.end()) return 4;
+  // float32 columns: one wave, whose CTAs fetch the next group while one is
+  // transformed (64 x 512^2 complex 184.3 -> 180.1 us per apply, 6 x 512^2 27.0
+  // -> 24.1, real 16 x 512^2 38.6 -> 35.0); float64 CTAs are small and even out
+  // over four (8 x 512^2 complex 203 against 206, 16 x 256^2 104 against 108)
+  if (it == g_waves.end()) return axis == 1 && !prec64 ? 1 : 4;
   return axis == 0 ? it->second.first : it->second.second;
 }
 
