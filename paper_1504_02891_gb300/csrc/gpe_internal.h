@@ -22,6 +22,16 @@ gpe_status cuda_fail(cudaError_t e, const char* what);
     if (e_ != cudaSuccess) return cuda_fail(e_, #call);  \
   } while (0)
 
+// Tables, cleared counters and other set-up data are written by plain copies and
+// memsets, that is on the legacy default stream, where they may still be on
+// their way when the call returns.  The streams that read them are other ones
+// (a plan's, a solve's, a batch group's, a refinement lane's), and non-blocking
+// streams do not wait for the legacy one: every create() ends with this wait.
+static inline gpe_status setup_done() {
+  GPE_CUDA(cudaStreamSynchronize(cudaStreamLegacy));
+  return GPE_OK;
+}
+
 // Host description of one grid (FP64 tables, §2).
 struct GridHost {
   int dim = 1;

@@ -227,7 +227,7 @@ gpe_status GridDev<T>::create(const GridHost& g) {
     max_blocks = std::max(max_blocks, fd_blocks);
   }
   max_blocks = std::max(max_blocks, 512 * g.nbatch);   // moments kernels
-  return GPE_OK;
+  return setup_done();
 }
 
 template <typename T>

@@ -241,7 +241,7 @@ gpe_status Scratch::create(size_t blocks, int nb) {
   GPE_CUDA(cudaMemset(results, 0, sizeof(double) * NQ * nb));
   GPE_CUDA(cudaMallocHost(&h_results, sizeof(double) * ((size_t)NQ * nb + 1)));
   h_results[(size_t)NQ * nb] = 0.0;
-  return GPE_OK;
+  return setup_done();
 }
 
 void Scratch::destroy() {

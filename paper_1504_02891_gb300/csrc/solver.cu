@@ -112,7 +112,7 @@ struct Level {
     h_err = reinterpret_cast<int*>(h + CB + RB);
     memset(h_ctl, 0, sizeof(Alg1Ctl));
     memset(h_rn, 0, sizeof(RNCtl));
-    return GPE_OK;
+    return setup_done();
   }
   void destroy() {
     for (int i = 0; i < 3; ++i)
@@ -167,6 +167,7 @@ unsigned long long* persist_debug_buffer(int* n) {
     if (cudaMallocHost(&g_pdbg_h, sizeof(unsigned long long) * 4 * PDBG_N) != cudaSuccess) return nullptr;
   }
   cudaMemset(g_pdbg, 0, sizeof(unsigned long long) * 4 * PDBG_N);
+  if (setup_done() != GPE_OK) return nullptr;
   *n = PDBG_N;
   return g_pdbg;
 }
@@ -1147,8 +1148,7 @@ gpe_status tune_cluster_share(const GridHost& gh, cudaStream_t st, int* best_kb,
     double ms_sum = 0.0;
     int nfe_sum = 0;
     for (int rep = 0; rep < 3 && s == GPE_OK; ++rep) {
-      if (cudaStreamSynchronize(st) != cudaSuccess ||
-          cudaMemcpy(L.xs[0], h.data(), L.bytes, cudaMemcpyHostToDevice) != cudaSuccess) {
+      if (cudaMemcpyAsync(L.xs[0], h.data(), L.bytes, cudaMemcpyHostToDevice, st) != cudaSuccess) {
         s = fail(GPE_ECUDA, "autotune start point");
         break;
       }
