@@ -59,6 +59,10 @@ struct Level {
   int p_grid[2] = {-1, -1};
   size_t p_smem[2] = {0, 0};
   float* d_omega = nullptr;   // Omega as float32 for the cluster engine
+  // host sides of level_set_problem's copies: an asynchronous copy may read
+  // pageable memory after the call has returned
+  std::vector<T> h_V;
+  float h_omega = 0.f;
 
   gpe_status create(const GridHost& gh) {
     g = gh;
@@ -1231,6 +1235,7 @@ struct BatchGroup {
   Alg1Ctl* ctl = nullptr;
   unsigned int* next = nullptr;
   std::vector<Alg1Ctl> hc;      // the instances' control blocks
+  std::vector<float> hv, hom;   // and potentials and Omegas: host sides of copies queued on st
   cudaStream_t st = nullptr;    // the groups' float32 stages run side by side
   std::chrono::steady_clock::time_point t0;
   ~BatchGroup() {
@@ -1251,14 +1256,15 @@ struct BatchGroup {
 
 // Point a level built for one problem of a group at another problem on the
 // same grid (extents, box, complexity): its potential, beta and Omega.  The
-// level's cached CUDA graphs captured the old operator and are dropped.
+// level's cached CUDA graphs captured the old operator and are dropped.  The
+// stream must have been waited for since the level's last problem was set.
 template <typename T>
 static gpe_status level_set_problem(Level<T>& L, const GridHost& gi, cudaStream_t st) {
   L.g.beta = gi.beta;
   L.g.omega = gi.omega;
-  std::vector<T> hv((size_t)L.M);
+  std::vector<T>& hv = L.h_V;
+  hv.resize((size_t)L.M);
   for (long long i = 0; i < L.M; ++i) hv[(size_t)i] = (T)gi.V[(size_t)i];
-  // (pageable: returns once the values are staged; ordered on the lane's stream)
   GPE_CUDA(cudaMemcpyAsync(L.d.V, hv.data(), sizeof(T) * hv.size(), cudaMemcpyHostToDevice, st));
   if (L.g.disc != GPE_FD) {
     for (int a = 0; a < 2 && a < L.g.dim; ++a) {
@@ -1273,8 +1279,8 @@ static gpe_status level_set_problem(Level<T>& L, const GridHost& gi, cudaStream_
     }
   }
   L.d.fd.omega = gi.omega;
-  const float om = (float)gi.omega;
-  GPE_CUDA(cudaMemcpyAsync(L.d_omega, &om, sizeof(float), cudaMemcpyHostToDevice, st));
+  L.h_omega = (float)gi.omega;
+  GPE_CUDA(cudaMemcpyAsync(L.d_omega, &L.h_omega, sizeof(float), cudaMemcpyHostToDevice, st));
   for (int i = 0; i < 3; ++i)
     if (L.chunk_exec[i]) {
       cudaGraphExecDestroy(L.chunk_exec[i]);
@@ -1312,8 +1318,10 @@ static gpe_status queue_batch_group(BatchGroup& B, const std::vector<GridHost>& 
   GPE_CUDA(cudaMalloc(&B.ctl, sizeof(Alg1Ctl) * n));
   GPE_CUDA(cudaMalloc(&B.next, sizeof(unsigned int)));
   // per-instance potential, Omega and control (alpha = beta / (2 h_vol))
-  std::vector<float> hv((size_t)M * n), hom(n);
+  std::vector<float>&hv = B.hv, &hom = B.hom;
   std::vector<Alg1Ctl>& hc = B.hc;
+  hv.resize((size_t)M * n);
+  hom.resize(n);
   hc.resize(n);
   for (int k = 0; k < n; ++k) {
     const GridHost& gi = gh[B.idx[k]];
