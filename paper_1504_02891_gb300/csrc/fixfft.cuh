@@ -351,7 +351,7 @@ struct LineFFT<double, LF> {
         for (int s = 0; s < 8; ++s) {
           const int m = j + s * TPL;
           const int p = m < (F >> 1) ? m : m - F;
-          const I2 c = fix_cmul<false>(mkI2(z[s].x, -z[s].y), __ldg(fine + (p & (2 * F - 1))));
+          const I2 c = fix_cmul<false>(mkI2(z[s].x, -z[s].y), ld_const(fine + (p & (2 * F - 1))));
           const bool nyq = m == (F >> 1);
           z[s] = mkI2(nyq ? 0 : (c.x + h) >> k, nyq ? 0 : (c.y + h) >> k);
         }

@@ -295,8 +295,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, fused_minb(LF)) k_fused2d(PassG
     // Both kinds of task share one copy of the line transform below: four
     // unrolled copies of it (y and x, forward and inverse) overflow the
     // instruction cache.  Every load of a task is issued before its first
-    // store (a store in between would hold the later loads back); read-only
-    // operands go through the non-coherent path.
+    // store (a store in between would hold the later loads back).
     C v[PPT];
     int ok = 1;
     long long cb = 0, rb = 0, ib = 0;
@@ -310,7 +309,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, fused_minb(LF)) k_fused2d(PassG
 #pragma unroll
         for (int s = 0; s < PPT; ++s) {
           const long long e = cb + (long long)(j + TPL * s) * n0c;
-          v[s] = sa * __ldg(ysrc0 + e) + sb * __ldg(ysrc1 + e);
+          v[s] = sa * __ldcg(ysrc0 + e) + sb * __ldcg(ysrc1 + e);
         }
 #pragma unroll
         for (int s = 0; s < PPT; ++s) yst[cb + (long long)(j + TPL * s) * n0c] = v[s];
@@ -320,8 +319,8 @@ __global__ void __launch_bounds__(FUSED_THREADS, fused_minb(LF)) k_fused2d(PassG
 #pragma unroll
         for (int s = 0; s < PPT; ++s) {
           const long long e = cb + (long long)(j + TPL * s) * n0c;
-          C a = __ldg(xc + e);
-          if (sc) a = a - __ldg(sc + e);
+          C a = __ldcg(xc + e);
+          if (sc) a = a - __ldcg(sc + e);
           v[s] = a;
         }
       }
@@ -348,21 +347,21 @@ __global__ void __launch_bounds__(FUSED_THREADS, fused_minb(LF)) k_fused2d(PassG
       ib = (long long)b * M;
       rb = ib + (long long)row0 * n0 + j;
       // the input: the trial point written by this launch's y-tasks (step
-      // on load), else read-only data
+      // on load), or a field of the kernels before
 #pragma unroll
       for (int s = 0; s < PPT; ++s) {
         if constexpr (CPLX) {
           const long long e = rb + TPL * s;
-          V a = yst ? __ldcg(xin + e) : __ldg(xin + e);
-          if (xsub) a = a - __ldg(xsub + e);
+          V a = __ldcg(xin + e);
+          if (xsub) a = a - __ldcg(xsub + e);
           v[s] = a;
         } else {
           const long long e = rb + TPL * s;
-          T a = yst ? __ldcg(xin + e) : __ldg(xin + e);
-          T c = yst ? __ldcg(xin + e + n0) : __ldg(xin + e + n0);
+          T a = __ldcg(xin + e);
+          T c = __ldcg(xin + e + n0);
           if (xsub) {
-            a -= __ldg(xsub + e);
-            c -= __ldg(xsub + e + n0);
+            a -= __ldcg(xsub + e);
+            c -= __ldcg(xsub + e + n0);
           }
           v[s].x = a;
           v[s].y = c;
@@ -422,21 +421,31 @@ __global__ void __launch_bounds__(FUSED_THREADS, fused_minb(LF)) k_fused2d(PassG
         T pacc[NQ];
 #pragma unroll
         for (int q = 0; q < NQ; ++q) pacc[q] = T(0);
+        const bool diff = epilogue_diff(E);
+        constexpr int NE = epi_batch<V, EPI>(NV);   // values whose operands are loaded ahead of their stores
+        auto at = [&](int q) -> long long { return rb + (long long)(q / PPT) * n0 + TPL * (q % PPT); };
 #pragma unroll
-        for (int q = 0; q < NV; ++q) {
-          const long long gi = rb + (long long)(q / PPT) * n0 + TPL * (q % PPT);
-          const C xs = stash[j + TPL * (q % PPT)];
-          V x, kin;
-          if constexpr (CPLX) {
-            x = xs;
-            kin = v[q];
-          } else {
-            x = (q < PPT) ? xs.x : xs.y;
-            kin = (q < PPT) ? v[q].x : v[q - PPT].y;
+        for (int q0 = 0; q0 < NV; q0 += NE) {
+          EpiOps<V, EPI> o[NE];
+#pragma unroll
+          for (int u = 0; u < NE; ++u) epilogue_load<T, CPLX, EPI, 1>(o[u], E, at(q0 + u));
+#pragma unroll
+          for (int u = 0; u < NE; ++u) {
+            const int q = q0 + u;
+            const long long gi = at(q);
+            const C xs = stash[j + TPL * (q % PPT)];
+            V x, kin;
+            if constexpr (CPLX) {
+              x = xs;
+              kin = v[q];
+            } else {
+              x = (q < PPT) ? xs.x : xs.y;
+              kin = (q < PPT) ? v[q].x : v[q - PPT].y;
+            }
+            const V lin = kin + ld_const(Vp + (gi - ib)) * x;
+            if constexpr (FPART) epilogue_apply<T, CPLX, EPI>(E, gi, x, lin, o[u], pacc, amax, diff);
+            else epilogue_apply<T, CPLX, EPI>(E, gi, x, lin, o[u], acc, amax, diff);
           }
-          const V lin = kin + __ldg(Vp + (gi - ib)) * x;
-          if constexpr (FPART) epilogue_point<T, CPLX, EPI, 2>(E, gi, x, lin, pacc, amax);
-          else epilogue_point<T, CPLX, EPI, 2>(E, gi, x, lin, acc, amax);
         }
         if constexpr (FPART) {
 #pragma unroll

@@ -175,14 +175,18 @@ __global__ void __launch_bounds__(lines_y_threads<T>(LF)) k_lines_y(PassGeom<T> 
   if (blockIdx.x < total) fetch(blockIdx.x);
   for (int gidx = blockIdx.x; gidx < total; gidx += gridDim.x) {
     const long long base = ebase(gidx);
+    C v[8], xkv[8];
+    if (xk) {   // ahead of the stores of the step
+#pragma unroll
+      for (int s = 0; s < 8; ++s) xkv[s] = __ldcg(xk + base + (long long)(j + s * TPL) * n0c);
+    }
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-    C v[8];
 #pragma unroll
     for (int s = 0; s < 8; ++s) {
       C a = pf0[s * NT + tid];
       if (src1) {
         const C b = pf1[s * NT + tid];
-        if (xk) a = sk * __ldg(xk + base + (long long)(j + s * TPL) * n0c) + sa * a + sb * b;
+        if (xk) a = sk * xkv[s] + sa * a + sb * b;
         else a = yst ? sa * a + sb * b : a - b;
         if (yst) yst[base + (long long)(j + s * TPL) * n0c] = a;
       }
@@ -314,18 +318,27 @@ __global__ void __launch_bounds__(lines_x_threads<T>(LF), lines_x_minb<T>(LF)) k
     sym.c1c = (CPLX && G.rcoord) ? G.c1 * G.rcoord[row0] : T(0);
     fft.apply(v, ex, par, sym);
     asm volatile("cp.async.wait_group %0;\n" ::"n"(0) : "memory");
+    const bool diff = epilogue_diff(E);
+    constexpr int NE = epi_batch<V, EPI>(NV);   // values whose operands are loaded ahead of their stores
 #pragma unroll
-    for (int q = 0; q < NV; ++q) {
-      const long long gi = gidx(grp, q);
-      V x = xs[(b * NV + q) * NT + tid];
-      if (xsub) x = x - xsub[gi];
-      V kin;
-      if constexpr (CPLX) kin = v[q];
-      else kin = (q < 8) ? v[q].x : v[q - 8].y;
-      if (accin) kin = kin + ea[q * NT + tid];
-      const V lin = kin + ev[q * NT + tid] * x;
-      if constexpr (FPART) epilogue_point<T, CPLX, EPI, 2>(E, gi, x, lin, pacc, amax);
-      else epilogue_point<T, CPLX, EPI, 2>(E, gi, x, lin, acc, amax);
+    for (int q0 = 0; q0 < NV; q0 += NE) {
+      EpiOps<V, EPI> o[NE];
+#pragma unroll
+      for (int u = 0; u < NE; ++u) epilogue_load<T, CPLX, EPI, 1>(o[u], E, gidx(grp, q0 + u));
+#pragma unroll
+      for (int u = 0; u < NE; ++u) {
+        const int q = q0 + u;
+        const long long gi = gidx(grp, q);
+        V x = xs[(b * NV + q) * NT + tid];
+        if (xsub) x = x - xsub[gi];
+        V kin;
+        if constexpr (CPLX) kin = v[q];
+        else kin = (q < 8) ? v[q].x : v[q - 8].y;
+        if (accin) kin = kin + ea[q * NT + tid];
+        const V lin = kin + ev[q * NT + tid] * x;
+        if constexpr (FPART) epilogue_apply<T, CPLX, EPI>(E, gi, x, lin, o[u], pacc, amax, diff);
+        else epilogue_apply<T, CPLX, EPI>(E, gi, x, lin, o[u], acc, amax, diff);
+      }
     }
     if constexpr (FPART) {
 #pragma unroll

@@ -333,25 +333,29 @@ __global__ void __launch_bounds__(axx_threads<T>(LF), axx_minb<T>(LF)) k_axis_x(
     if constexpr (KIND == LK_SINE) mirror_odd<T, LF>(v, ex, par, j);
     sym.c1c = (CPLX && G.rcoord && r0 < rows) ? G.c1 * G.rcoord[r0 % G.n1] : T(0);
     fft.apply(v, ex, par, sym);
-    auto point = [&](int q, V x, V aq, T pv) {
-      V kin;
-      if constexpr (CPLX) kin = v[q];
-      else kin = q < NP ? v[q % NP].x : v[q % NP].y;
+    // v becomes the linear part: + accumulator + V x
+    auto part = [&](int q) -> V& {
+      if constexpr (CPLX) return v[q];
+      else return q < NP ? v[q % NP].x : v[q % NP].y;
+    };
+    auto value = [&](int q) -> V {
+      if constexpr (REGS) return xv[q];
+      else return es[q * NT + tid];
+    };
+    auto add_lin = [&](int q, V aq, T pv) {
+      V kin = part(q);
       if (REGS || accin) kin = kin + aq;
-      const V lin = kin + pv * x;
-      // (read-only loads of the other vectors: plain ones would each wait for
-      // the store before it)
-      epilogue_point<T, CPLX, EPI, 2>(E, ibase + at(q), x, lin, acc, amax);
+      part(q) = kin + pv * value(q);
     };
     if constexpr (REGS) {
 #pragma unroll
       for (int q = 0; q < NV; ++q)
-        if (has(q)) point(q, xv[q], av[q], vv[q]);
+        if (has(q)) add_lin(q, av[q], vv[q]);
     } else if (slots) {
       cp_async_wait_all();
 #pragma unroll
       for (int q = 0; q < NV; ++q)
-        if (has(q)) point(q, es[q * NT + tid], accin ? es[(NV + q) * NT + tid] : vzero<V>(), ev[q * NT + tid]);
+        if (has(q)) add_lin(q, accin ? es[(NV + q) * NT + tid] : vzero<V>(), ev[q * NT + tid]);
     } else {
       constexpr int NE = NV < 8 ? NV : 8;   // values whose operands are in flight together
 #pragma unroll
@@ -363,13 +367,26 @@ __global__ void __launch_bounds__(axx_threads<T>(LF), axx_minb<T>(LF)) k_axis_x(
           ac[u] = vzero<V>();
           pc[u] = T(0);
           if (!has(q0 + u)) continue;
-          if (accin) ac[u] = ldv<2>(accin + ibase + at(q0 + u));
-          pc[u] = ldv<2>(Vp + at(q0 + u));
+          if (accin) ac[u] = __ldcg(accin + ibase + at(q0 + u));
+          pc[u] = ld_const(Vp + at(q0 + u));
         }
 #pragma unroll
         for (int u = 0; u < NE; ++u)
-          if (has(q0 + u)) point(q0 + u, es[(q0 + u) * NT + tid], ac[u], pc[u]);
+          if (has(q0 + u)) add_lin(q0 + u, ac[u], pc[u]);
       }
+    }
+    const bool diff = epilogue_diff(E);
+    constexpr int NB = epi_batch<V, EPI>(NV);   // values whose vectors are loaded ahead of their stores
+#pragma unroll
+    for (int q0 = 0; q0 < NV; q0 += NB) {
+      EpiOps<V, EPI> o[NB];
+#pragma unroll
+      for (int u = 0; u < NB; ++u)
+        if (has(q0 + u)) epilogue_load<T, CPLX, EPI, 1>(o[u], E, ibase + at(q0 + u));
+#pragma unroll
+      for (int u = 0; u < NB; ++u)
+        if (has(q0 + u))
+          epilogue_apply<T, CPLX, EPI>(E, ibase + at(q0 + u), value(q0 + u), part(q0 + u), o[u], acc, amax, diff);
     }
   }
   if (EPI == EPI_HESS || D.nq == 0) return;

@@ -815,7 +815,11 @@ static __device__ void rn_control(RNCtl* c, const double* r) {
 // the one before it drains, loads its constant tables, and waits
 // (griddepcontrol.wait) for that kernel's completion and memory before it
 // touches anything else.  Every CTA of every such kernel executes the wait
-// before it can return, so completion is transitive along the stream.  Launches
+// before it can return, so completion is transitive along the stream.  The wait
+// orders ordinary loads (ld, ld.cg, cp.async).  The read-only path is for data
+// that nobody writes while the kernel is resident, and that is longer than its
+// own work here: fields, accumulators and sums are never read through it, only
+// the tables and potentials of a plan (ld_const).  Launches
 // being captured keep plain edges: the solver's graphs of 16 iterations ran 2%
 // slower with programmatic ones (64^3: 14.9 against 14.6 ms a solve).  Measured:
 // 127^3 Hessian-vector float32 59 -> 50 us, 64^3 -> 128^3 transfer 32 -> 24 us,
@@ -842,14 +846,14 @@ static cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, int threads, size
 // ----------------------------------------------------------------- coherent loads
 // Inside a persistent launch, data written by other CTAs during the same launch
 // must bypass the (non-coherent) L1: ld.global.cg.
-// COH = 2: data that no thread writes during the launch, loaded through the
-// read-only path (the compiler may then issue the loads ahead of earlier
-// stores, which it must not do for plain loads of possibly aliasing arrays).
 template <int COH, typename X> __device__ __forceinline__ X ldv(const X* p) {
+  static_assert(COH == 0 || COH == 1, "plain or coherent in L2");
   if constexpr (COH == 1) return __ldcg(p);
-  else if constexpr (COH == 2) return __ldg(p);
   else return *p;
 }
+// The read-only path: potentials and tables, written when a plan or a level is
+// set up and by no kernel.
+template <typename X> __device__ __forceinline__ X ld_const(const X* p) { return __ldg(p); }
 template <int COH, typename X> __device__ __forceinline__ X rdc(const X& r) {
   if constexpr (COH == 1) return *(const volatile X*)&r;
   else return r;
@@ -867,43 +871,67 @@ struct EpiCtx {
   T nl, shift, lin_scale, th_c, delta, thk;
 };
 
-// One point of the objective passes (F, W, WS) with the current point's values
-// xc, gc at hand; base and gk are constant during a launch (read with COH).
-// diff: there is a current point.  A run's first evaluation has none and its
-// control reads no difference sum (slots Q_SS.. and Q_MAX); in float64 they are
-// half of the 36 operations a point, of which an SM sub-partition issues one
-// warp's in 64 clocks: they were 37 of the 80 thousand cycles of the 256^2 real
-// x-kernel (49 -> 44.5 us without the differences).
-template <typename T, bool CPLX, int EPI, int COH = 2, typename A>
-__device__ __forceinline__ void epilogue_values(const EpiCtx<T, CPLX>& E, long long gi, typename VT<T, CPLX>::V x,
-                                                typename VT<T, CPLX>::V lin, typename VT<T, CPLX>::V xc,
-                                                typename VT<T, CPLX>::V gc, A (&acc)[NQ], T& amax, bool diff = true);
-
-template <typename T, bool CPLX, int EPI, int COH = 0, typename A>
-__device__ __forceinline__ void epilogue_point(const EpiCtx<T, CPLX>& E, long long gi,
-                                               typename VT<T, CPLX>::V x,
-                                               typename VT<T, CPLX>::V lin, A (&acc)[NQ], T& amax) {
+// The vectors an epilogue reads at a point besides x and its linear part: HESS
+// psi; F X_cur, G_cur; W those and X^k; WS those and P_k; RATIO X^k, G_k.  They
+// are values here, so that a kernel can load those of several points before
+// the first store (the compiler has to keep a load behind a store that may
+// alias it, so each point would wait for the one before).
+constexpr __host__ __device__ int epi_nops(int epi) {
+  return epi == EPI_HESS ? 1 : (epi == EPI_F || epi == EPI_RATIO) ? 2 : epi == EPI_W ? 3 : epi == EPI_WS ? 4 : 0;
+}
+template <typename V, int EPI> struct EpiOps {
+  V v[epi_nops(EPI) > 0 ? epi_nops(EPI) : 1];
+};
+// Points whose operands are held together: at most 16 registers.
+template <typename V, int EPI> constexpr __host__ __device__ int epi_batch(int nv) {
+  int n = nv;
+  while (n > 1 && n * epi_nops(EPI) * (int)sizeof(V) > 64) n /= 2;
+  return n;
+}
+template <typename T, bool CPLX, int EPI, int COH>
+__device__ __forceinline__ void epilogue_load(EpiOps<typename VT<T, CPLX>::V, EPI>& o, const EpiCtx<T, CPLX>& E,
+                                              long long gi) {
   using V = typename VT<T, CPLX>::V;
-  if (EPI == EPI_GRAD) {
+  if constexpr (EPI == EPI_HESS) {
+    o.v[0] = ldv<COH>(E.base + gi);
+  } else if constexpr (EPI == EPI_RATIO) {
+    o.v[0] = ldv<COH>(E.base + gi);
+    o.v[1] = ldv<COH>(E.gk + gi);
+  } else if constexpr (epi_nops(EPI) > 0) {
+    o.v[0] = E.xc ? ldv<COH>(E.xc + gi) : vzero<V>();
+    o.v[1] = E.gc ? ldv<COH>(E.gc + gi) : vzero<V>();
+    if constexpr (EPI == EPI_W || EPI == EPI_WS) o.v[2] = ldv<COH>(E.base + gi);
+    if constexpr (EPI == EPI_WS) o.v[3] = ldv<COH>(E.gk + gi);
+  }
+}
+
+// One point: output and sums.  diff (objective passes): there is a current
+// point.  A run's first evaluation has none and its control reads no difference
+// sum (slots Q_SS.. and Q_MAX); in float64 they are half of the 36 operations a
+// point, of which an SM sub-partition issues one warp's in 64 clocks: they were
+// 37 of the 80 thousand cycles of the 256^2 real x-kernel (49 -> 44.5 us without
+// the differences).
+template <typename T, bool CPLX, int EPI, typename A>
+__device__ __forceinline__ void epilogue_apply(const EpiCtx<T, CPLX>& E, long long gi, typename VT<T, CPLX>::V x,
+                                               typename VT<T, CPLX>::V lin,
+                                               const EpiOps<typename VT<T, CPLX>::V, EPI>& o, A (&acc)[NQ], T& amax,
+                                               bool diff) {
+  using V = typename VT<T, CPLX>::V;
+  if constexpr (EPI == EPI_GRAD) {
     const T x2 = tre(x, x);
     if (E.out) E.out[gi] = lin + (E.nl * x2) * x;
     acc_add(acc[0], tre(x, lin));
     acc_add(acc[1], x2 * x2);
     acc_add(acc[2], x2);
-  } else if (EPI == EPI_HESS) {
-    const V p = ldv<COH>(E.base + gi);
+  } else if constexpr (EPI == EPI_HESS) {
+    const V p = o.v[0];
     const T p2 = tre(p, p);
     const T R = tre(p, x);
     // gathered by x and p: 12 operations a complex point instead of 18 (float64 issues 2 a clock)
     E.out[gi] = lin + (E.nl * p2 + E.shift) * x + (T(2) * E.nl * R) * p;
-  } else if (EPI == EPI_F || EPI == EPI_W || EPI == EPI_WS) {
-    const V xc = E.xc ? ldv<COH>(E.xc + gi) : vzero<V>();
-    const V gc = E.gc ? ldv<COH>(E.gc + gi) : vzero<V>();
-    epilogue_values<T, CPLX, EPI, COH>(E, gi, x, lin, xc, gc, acc, amax, sizeof(T) == 4 || E.xc != nullptr);
-  } else if (EPI == EPI_RATIO) {
+  } else if constexpr (EPI == EPI_RATIO) {
     const V d = x;
-    const V xk = ldv<COH>(E.base + gi);
-    const V gk = ldv<COH>(E.gk + gi);
+    const V xk = o.v[0], gk = o.v[1];
     const T x2 = tre(xk, xk);
     const V ax = gk - (T(4) * E.nl * x2) * xk;
     const V z = xk + d;
@@ -916,21 +944,13 @@ __device__ __forceinline__ void epilogue_point(const EpiCtx<T, CPLX>& E, long lo
     acc_add(acc[R_DD], d2);
     acc_add(acc[R_GD], tre(gk, d));
     amax = fmax(amax, d2);
-  }
-}
-
-template <typename T, bool CPLX, int EPI, int COH, typename A>
-__device__ __forceinline__ void epilogue_values(const EpiCtx<T, CPLX>& E, long long gi, typename VT<T, CPLX>::V x,
-                                                typename VT<T, CPLX>::V lin, typename VT<T, CPLX>::V xc,
-                                                typename VT<T, CPLX>::V gc, A (&acc)[NQ], T& amax, bool diff) {
-  using V = typename VT<T, CPLX>::V;
-  if (EPI == EPI_F || EPI == EPI_W) {
+  } else if constexpr (EPI == EPI_F || EPI == EPI_W) {
     const V y = x;
     V g;
-    if (EPI == EPI_F) {
+    if constexpr (EPI == EPI_F) {
       g = E.lin_scale * lin + (T(4) * E.nl * tre(y, y)) * y;
     } else {
-      const V xk = ldv<COH>(E.base + gi);
+      const V xk = o.v[2];
       const V dd = y - xk;
       const T x2 = tre(xk, xk);
       const T R = tre(xk, dd);
@@ -949,6 +969,7 @@ __device__ __forceinline__ void epilogue_values(const EpiCtx<T, CPLX>& E, long l
     acc_add(acc[Q_Q], tre(q, q));
     acc_add(acc[Q_QY], tre(q, y));
     if (!diff) return;
+    const V xc = o.v[0], gc = o.v[1];
     const V s = y - xc;
     const V v = (g - gc) - E.th_c * s;
     const T s2 = tre(s, s);
@@ -965,13 +986,12 @@ __device__ __forceinline__ void epilogue_values(const EpiCtx<T, CPLX>& E, long l
     if (EPI == EPI_F) df -= E.nl * tre(s, y + xc) * s2;
     acc_add(acc[Q_DF], df);
     amax = fmax(amax, s2);
-  } else if (EPI == EPI_WS) {
+  } else if constexpr (EPI == EPI_WS) {
     // difference form (the unknown y is D = X - X^k): G^ = P_k + H_k D +
     // (delta - theta_k) D, objective Re<P_k, D> + theta_k Re<X^k, D> +
     // 1/2 Re<D, H_k D> + delta/2 |D|^2, moments of X = X^k + D
     const V y = x;
-    const V xk = ldv<COH>(E.base + gi);
-    const V pk = ldv<COH>(E.gk + gi);
+    const V xc = o.v[0], gc = o.v[1], xk = o.v[2], pk = o.v[3];
     const T x2 = tre(xk, xk), R = tre(xk, y);
     const V hD = E.lin_scale * lin + (T(4) * E.nl) * (x2 * y + (T(2) * R) * xk);
     const V gh = pk + hD + (E.delta - E.thk) * y;
@@ -995,6 +1015,18 @@ __device__ __forceinline__ void epilogue_values(const EpiCtx<T, CPLX>& E, long l
     acc_add(acc[Q_DF], tre(s, q) - T(0.5) * tre(s, v));   // the model is quadratic: trapezoid exact
     amax = fmax(amax, s2);
   }
+}
+
+// The first evaluation of a float64 run leaves out the difference sums.
+template <typename T, bool CPLX> __device__ __forceinline__ bool epilogue_diff(const EpiCtx<T, CPLX>& E) {
+  return sizeof(T) == 4 || E.xc != nullptr;
+}
+template <typename T, bool CPLX, int EPI, int COH = 0, typename A>
+__device__ __forceinline__ void epilogue_point(const EpiCtx<T, CPLX>& E, long long gi, typename VT<T, CPLX>::V x,
+                                               typename VT<T, CPLX>::V lin, A (&acc)[NQ], T& amax) {
+  EpiOps<typename VT<T, CPLX>::V, EPI> o;
+  epilogue_load<T, CPLX, EPI, COH>(o, E, gi);
+  epilogue_apply<T, CPLX, EPI>(E, gi, x, lin, o, acc, amax, epilogue_diff(E));
 }
 
 template <typename T, bool CPLX, int EPI, int COH = 0>
@@ -1412,7 +1444,7 @@ __global__ void __launch_bounds__(NTHREADS) k_fd(FDGeom G, const T* __restrict__
       }
     }
     if constexpr (!F64) lin = lin + D.V[li] * x;
-    epilogue_point<T, CPLX, EPI, 2>(E, base + li, x, lin, acc, amax);
+    epilogue_point<T, CPLX, EPI>(E, base + li, x, lin, acc, amax);
   }
   if (EPI == EPI_HESS || D.nq == 0) return;
   run_control<T>(D, reduce_partials(acc, amax, D.nq, D.partials, D.results, D.ticket, G.tiles));

@@ -223,7 +223,7 @@ __global__ void __launch_bounds__(pl_threads<LF>()) k_alg1_lines(PersistLinesArg
         if (has(q)) {
           xv[q] = __ldcg(yt + at(q));
           av[q] = __ldcg(acc + at(q));
-          vv[q] = __ldg(Vp + at(q));
+          vv[q] = ld_const(Vp + at(q));
         }
       }
       C v[8];
@@ -259,7 +259,14 @@ __global__ void __launch_bounds__(pl_threads<LF>()) k_alg1_lines(PersistLinesArg
         if constexpr (CPLX) kin = v[q];
         else kin = q < NP ? v[q % NP].x : v[q % NP].y;
         const V lin = (kin + av[q]) + vv[q] * xv[q];
-        epilogue_values<T, CPLX, EPI>(E, at(q), xv[q], lin, xcv[q], gcv[q], sums, amax);
+        EpiOps<V, EPI> o;
+        o.v[0] = xcv[q];
+        o.v[1] = gcv[q];
+        if constexpr (EPI == EPI_WS) {   // constant during the launch
+          o.v[2] = __ldg(E.base + at(q));
+          o.v[3] = __ldg(E.gk + at(q));
+        }
+        epilogue_apply<T, CPLX, EPI>(E, at(q), xv[q], lin, o, sums, amax, true);
       }
     }
     block_partial(sums, amax, NQ, P.D.partials + (size_t)blockIdx.x * NQ);

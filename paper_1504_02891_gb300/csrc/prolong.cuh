@@ -29,7 +29,7 @@ __device__ __forceinline__ void midpoints(const LineFFT<float, LF>& fft, float2 
     const int m = fft.j + s * TPL;
     const int p = m < (F >> 1) ? m : m - F;
     // conj(v e^{i pi p / F}) / F = conj(v) e^{-2 pi i p / (2F)} / F
-    const float2 w = __ldg(fine + (p & (2 * F - 1)));
+    const float2 w = ld_const(fine + (p & (2 * F - 1)));
     const float sc = m == (F >> 1) ? 0.f : 1.f / F;
     v[s] = cmul(make_float2(sc * v[s].x, -sc * v[s].y), w);
   }
