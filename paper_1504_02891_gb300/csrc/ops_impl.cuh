@@ -1358,10 +1358,15 @@ __global__ void __launch_bounds__(NTHREADS) k_alg1_persist(PersistArgs<T> P) {
 // ----------------------------------------------------------------- finite differences
 // H_lin of §2.1 per axis (3/5/7-point, zero Dirichlet values outside) with the
 // central-difference rotation term, then the same epilogue as the spectral pass.
-// Float64 is bound by the float64 pipe (2 operations a clock and SM): the
-// diagonal is one coefficient per point, V + sum 1/h^2, each axis adds one
-// addition and one multiply-add, and the CTAs are few (two per SM) because a
-// warp's reduction costs as much as two of its points.
+// Float64 is bound by the float64 pipe (2 operations a clock and SM): each axis
+// is one addition and two multiply-adds, (x - (x- + x+)/2) / h^2, and the CTAs
+// are few (two per SM) because a warp's reduction costs as much as two of its
+// points.  The difference is taken before it is scaled: its rounding is that of
+// the neighbours' sum alone.  With one diagonal (V + sum 1/h^2) x for all axes
+// the kernel was two operations a point and 4 us shorter (149 x 100 x 76: 71.2
+// against 75.3 us), but its error 2 to 2.5 times as large on smooth states of
+// two and three dimensions (against extended precision; scaling each x and
+// neighbours' sum by itself lies between).
 template <typename T, bool CPLX, int EPI>
 __global__ void __launch_bounds__(NTHREADS) k_fd(FDGeom G, const T* __restrict__ rx, const T* __restrict__ ry,
                                                 PassData<T> D) {
@@ -1386,8 +1391,6 @@ __global__ void __launch_bounds__(NTHREADS) k_fd(FDGeom G, const T* __restrict__
   if (xsub) xsub += base;
   const T a0 = (T)G.ih2[0], a1 = (T)G.ih2[1], a2 = (T)G.ih2[2];
   constexpr bool F64 = sizeof(T) == 8;
-  const T adiag = a0 + a1 + a2;                  // (axes beyond dim have ih2 = 0)
-  const T h0 = T(-0.5) * a0, h1 = T(-0.5) * a1, h2 = T(-0.5) * a2;
   const unsigned int n0 = G.n0, n1 = G.n1, n2 = G.n2, s2 = n0 * n1, M = (unsigned int)G.M;
   const unsigned int step = (unsigned int)G.tiles * blockDim.x;
   for (unsigned int li = (unsigned int)tb * blockDim.x + threadIdx.x; li < M; li += step) {
@@ -1403,18 +1406,18 @@ __global__ void __launch_bounds__(NTHREADS) k_fd(FDGeom G, const T* __restrict__
     V xp = i0 < n0 - 1 ? ld(li + 1) : vzero<V>();
     V dx = vzero<V>(), dy = vzero<V>(), lin;
     if constexpr (F64) {
-      lin = (adiag + D.V[li]) * x + h0 * (xm + xp);
+      lin = a0 * (x + T(-0.5) * (xm + xp));
       if constexpr (CPLX) dx = xp - xm;
       if (G.dim >= 2) {
         V ym = i1 > 0 ? ld(li - n0) : vzero<V>();
         V yp = i1 < n1 - 1 ? ld(li + n0) : vzero<V>();
-        lin = lin + h1 * (ym + yp);
+        lin = lin + a1 * (x + T(-0.5) * (ym + yp));
         if constexpr (CPLX) dy = yp - ym;
       }
       if (G.dim >= 3) {
         V zm = i2 > 0 ? ld(li - s2) : vzero<V>();
         V zp = i2 < n2 - 1 ? ld(li + s2) : vzero<V>();
-        lin = lin + h2 * (zm + zp);
+        lin = lin + a2 * (x + T(-0.5) * (zm + zp));
       }
     } else {
       lin = (a0) * x - (T(0.5) * a0) * (xm + xp);
@@ -1443,7 +1446,7 @@ __global__ void __launch_bounds__(NTHREADS) k_fd(FDGeom G, const T* __restrict__
         lin = lin + iw;
       }
     }
-    if constexpr (!F64) lin = lin + D.V[li] * x;
+    lin = lin + D.V[li] * x;
     epilogue_point<T, CPLX, EPI>(E, base + li, x, lin, acc, amax);
   }
   if (EPI == EPI_HESS || D.nq == 0) return;
