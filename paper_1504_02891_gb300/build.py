@@ -19,7 +19,7 @@ BUILD = os.path.join(ROOT, "_build", "gpe")
 LIB = os.path.join(PKG, "libgpe.so")
 SOURCES = ["ops_f32.cu", "ops_f64.cu", "plan.cu", "solver.cu", "noalloc.cu", "cluster.cu", "lines2d_f32.cu", "lines2d_f64.cu",
            "lines3_f32_a.cu", "lines3_f32_b.cu", "lines3_f32_c.cu", "lines3_f64_a.cu", "lines3_f64_b.cu", "lines3_f64_c.cu",
-           "persist_lines.cu", "pass_f32_acc.cu", "pass_f32_grad.cu", "certificate.cu", "autotune.cu", "probe.cu"]
+           "persist_lines.cu", "pass_f32_acc.cu", "pass_f32_grad.cu", "certificate.cu", "autotune.cu", "probe.cu", "device_limits.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
          "--expt-relaxed-constexpr", "-I", os.path.join(ROOT, "include")]

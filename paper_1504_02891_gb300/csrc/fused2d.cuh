@@ -553,11 +553,12 @@ static gpe_status launch_fused2d_t(const GridHost& g, const GridDev<T>& d, const
   PassData<T> Df = D;
   Df.step_on_load = step_first ? 1 : 0;
   const size_t smem = fused_smem<T, LF>();
-  static const KernelShape sh = kernel_shape((const void*)k_fused2d<T, CPLX, EPI, LF, PK>, FUSED_THREADS, smem);
-  GPE_CUDA(sh.e);
+  static KernelShape shape;
+  int occ = 0;
+  GPE_CUDA(kernel_shape(shape, (const void*)k_fused2d<T, CPLX, EPI, LF, PK>, FUSED_THREADS, smem, &occ));
   const long long ntask = (long long)nb * (FA.NY + FA.NX);
   const long long wpc = FUSED_THREADS / 32;
-  const int grid = (int)std::max<long long>(1, std::min<long long>((ntask + wpc - 1) / wpc, (long long)sh.occ * num_sms()));
+  const int grid = (int)std::max<long long>(1, std::min<long long>((ntask + wpc - 1) / wpc, (long long)occ * num_sms()));
   // S: about twice the warps in flight over the y-tasks per instance
   // (measured: 64 x 256^2 complex 87 -> 76 us per apply against once)
   FA.skew = (int)std::min<long long>(nb, (FUSED_SKEW * (long long)grid * wpc + FA.NY - 1) / FA.NY + 1);

@@ -6,6 +6,7 @@
 #include <stdlib.h>
 #include <string>
 #include <vector>
+#include "device_limits.h"
 #include "gpe_kernels.cuh"
 #include "../../include/gpe.h"
 
@@ -212,18 +213,6 @@ struct ProfScope {
   ~ProfScope();
 };
 const char* kernel_name(const char* base, int f64, int cplx, int epi, long long points = -1);
-
-// Dynamic shared memory a kernel may use and the CTAs of that shape per SM,
-// looked up once (a function-local static of the launcher).
-struct KernelShape {
-  cudaError_t e;
-  int occ;
-};
-KernelShape kernel_shape(const void* fn, int threads, size_t smem);
-// Raise a kernel's dynamic shared memory limit to at least `bytes` (never
-// lowered: other threads may be launching it with more).
-cudaError_t raise_smem(const void* fn, size_t bytes);
-int num_sms();
 
 inline size_t elem_size(int prec, int cplx) { return (prec == GPE_F64 ? 8 : 4) * (cplx ? 2 : 1); }
 

@@ -364,11 +364,12 @@ static gpe_status launch_lines_x(const GridDev<T>& d, const PassData<T>& Dx, int
   const size_t vsz = sizeof(T) * (CPLX ? 2 : 1);
   const size_t smem = ((size_t)(1 << LF0) + 2 * (size_t)NL * LineFFT<T, LF0>::P) * sizeof(C) +
                       3 * (size_t)NV * NTX * vsz + (size_t)NV * NTX * sizeof(T);
-  static const KernelShape sh = kernel_shape((const void*)k_lines_x<T, CPLX, EPI, LF0>, NTX, smem);
-  GPE_CUDA(sh.e);
+  static KernelShape shape;
+  int occ = 0;
+  GPE_CUDA(kernel_shape(shape, (const void*)k_lines_x<T, CPLX, EPI, LF0>, NTX, smem, &occ));
   // a few resident waves in all (4, or the measured choice), at most the
   // reduction scratch's capacity
-  const long long want = (long long)tuned_waves(0, sizeof(T) == 8, CPLX, gx.n0, gx.n1, nbatch) * sh.occ * num_sms();
+  const long long want = (long long)tuned_waves(0, sizeof(T) == 8, CPLX, gx.n0, gx.n1, nbatch) * occ * num_sms();
   int tiles = groups;
   while (tiles > 1 && (long long)tiles * nbatch > want) tiles = (tiles + 1) / 2;
   while (tiles > 1 && (long long)tiles * nbatch > d.max_blocks) tiles = (tiles + 1) / 2;
@@ -400,10 +401,11 @@ static gpe_status launch_lines2d_t(const GridDev<T>& d, const PassData<T>& D, in
     Dy.nq = 0;
     Dy.control = 0;
     const size_t smem = ((size_t)(1 << LF1) * (1 + 2 * CW) + 16 * (size_t)YT) * sizeof(C);
-    static const KernelShape sh = kernel_shape((const void*)k_lines_y<T, CPLX, LF1>, YT, smem);
-    GPE_CUDA(sh.e);
+    static KernelShape shape;
+    int occ = 0;
+    GPE_CUDA(kernel_shape(shape, (const void*)k_lines_y<T, CPLX, LF1>, YT, smem, &occ));
     const int total = nbatch * colgroups;
-    const int grid = std::min(total, tuned_waves(1, sizeof(T) == 8, CPLX, gx.n0, gx.n1, nbatch) * sh.occ * num_sms());
+    const int grid = std::min(total, tuned_waves(1, sizeof(T) == 8, CPLX, gx.n0, gx.n1, nbatch) * occ * num_sms());
     ProfScope ps(kernel_name("linesy", sizeof(T) == 8, CPLX, EPI_ACC, gx.M * nbatch), st);
     GPE_CUDA(launch_pdl(k_lines_y<T, CPLX, LF1>, grid, YT, smem, st, gy, Dy, colgroups, total));
   }

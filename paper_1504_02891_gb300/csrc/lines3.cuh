@@ -402,8 +402,9 @@ static gpe_status launch_axis_s_t(const GridDev<T>& d, int axis, const PassData<
   const PassGeom<T>& G = d.geom[axis];
   constexpr int CW = axs_cw<T>(LF), NT = axs_threads<T>(LF);
   const size_t smem = (size_t)FFT::F * sizeof(typename FFT::Tw) + 2 * (size_t)FFT::F * CW * sizeof(typename FFT::X);
-  static const cudaError_t allowed = raise_smem((const void*)k_axis_s<T, KIND, LF>, smem);
-  GPE_CUDA(allowed);
+  static KernelShape shape;
+  int occ = 0;
+  GPE_CUDA(kernel_shape(shape, (const void*)k_axis_s<T, KIND, LF>, NT, smem, &occ));
   const int width = axis == 1 ? G.n0 : G.n0 * G.n1;
   const int planes = nbatch * (axis == 1 ? G.n2 : 1);
   const int cols = KIND == LK_CPLX ? CW : 2 * CW;
@@ -423,10 +424,10 @@ static gpe_status launch_axis_x_t(const GridDev<T>& d, const PassData<T>& D, int
   const size_t base = (size_t)FFT::F * sizeof(typename FFT::Tw) + 2 * (size_t)NL * FFT::P * sizeof(typename FFT::X);
   const size_t few = base + (sizeof(T) == 8 ? (size_t)NV * NT * vsz : 0);
   const size_t all = base + (sizeof(T) == 8 ? (size_t)NV * NT * (2 * vsz + sizeof(T)) : 0);
-  static const KernelShape sf = kernel_shape((const void*)k_axis_x<T, KIND, EPI, LF>, NT, few);
-  static const KernelShape sa = kernel_shape((const void*)k_axis_x<T, KIND, EPI, LF>, NT, all);
-  GPE_CUDA(sf.e);
-  GPE_CUDA(sa.e);
+  static KernelShape sf, sa;
+  int occ_few = 0, occ_all = 0;
+  GPE_CUDA(kernel_shape(sf, (const void*)k_axis_x<T, KIND, EPI, LF>, NT, few, &occ_few));
+  GPE_CUDA(kernel_shape(sa, (const void*)k_axis_x<T, KIND, EPI, LF>, NT, all, &occ_all));
   const long long rows = G.M / G.len;
   const long long lines = KIND == LK_CPLX ? rows : (rows + 1) / 2;
   const int groups = (int)((lines + NL - 1) / NL);
@@ -436,13 +437,12 @@ static gpe_status launch_axis_x_t(const GridDev<T>& d, const PassData<T>& D, int
   // real Fourier gradient 165 -> 147 us, 127^3 sine gradient 208.4 -> 206.5 and
   // Hessian-vector 188.6 -> 186.2; at 2.2 waves, four 64^3 complex gradients,
   // 151 against 153, at 1.6, three 64^3 sine gradients, 114 against 122)
-  const int slots = sizeof(T) == 8 && 2LL * groups * nbatch <= 5LL * sa.occ * num_sms();
-  const KernelShape& sh = slots ? sa : sf;
+  const int slots = sizeof(T) == 8 && 2LL * groups * nbatch <= 5LL * occ_all * num_sms();
   const size_t smem = slots ? all : few;
   // one resident wave (each CTA pays its tables and a reduction of its sums; a
   // CTA per group took 47.8 us for the 127^3 Hessian-vector product, this 45.6),
   // within the reduction scratch
-  long long cap = std::min<long long>((long long)sh.occ * num_sms(), d.max_blocks);
+  long long cap = std::min<long long>((long long)(slots ? occ_all : occ_few) * num_sms(), d.max_blocks);
   const int tiles = (int)std::max<long long>(1, std::min<long long>(groups, std::max<long long>(cap / nbatch, 1)));
   if ((long long)tiles * nbatch > d.max_blocks) return fail(GPE_EINVAL, "reduction scratch too small");
   ProfScope ps(kernel_name("axis_x", sizeof(T) == 8, KIND == LK_CPLX, EPI, G.M * nbatch), st);

@@ -288,8 +288,9 @@ static gpe_status launch_alg1_lines_t(PersistLinesArgs& P, int* grid_only, cudaS
   using FFT = LineFFT<float, LF>;
   constexpr int NT = pl_threads<LF>(), NL = NT / FFT::TPL, CW = NL;
   const size_t smem = ((size_t)FFT::F + 2 * std::max((size_t)FFT::F * CW, (size_t)NL * FFT::P)) * sizeof(float2);
-  static const KernelShape sh = kernel_shape((const void*)k_alg1_lines<KIND, EPI, LF>, NT, smem);
-  GPE_CUDA(sh.e);
+  static KernelShape shape;
+  int occ = 0;
+  GPE_CUDA(kernel_shape(shape, (const void*)k_alg1_lines<KIND, EPI, LF>, NT, smem, &occ));
   int most = 1;
   for (int a = 0; a < P.dim; ++a) {
     const PassGeom<float>& G = P.G[a];
@@ -304,7 +305,7 @@ static gpe_status launch_alg1_lines_t(PersistLinesArgs& P, int* grid_only, cudaS
     }
     most = std::max(most, P.total[a]);
   }
-  const int grid = std::min(most, sh.occ * num_sms());
+  const int grid = std::min(most, occ * num_sms());
   if (grid_only) {
     *grid_only = grid;
     return GPE_OK;

@@ -86,36 +86,6 @@ static void prof_clear() {
   g_recs.clear();
 }
 
-KernelShape kernel_shape(const void* fn, int threads, size_t smem) {
-  KernelShape k{raise_smem(fn, smem), 1};
-  if (k.e == cudaSuccess) k.e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&k.occ, fn, threads, smem);
-  if (k.occ < 1) k.occ = 1;
-  return k;
-}
-
-cudaError_t raise_smem(const void* fn, size_t bytes) {
-  static std::mutex mu;
-  static std::map<std::pair<int, const void*>, size_t> allowed;   // (device, kernel)
-  int dev = 0;
-  cudaGetDevice(&dev);
-  std::lock_guard<std::mutex> lk(mu);
-  size_t& have = allowed[{dev, fn}];
-  if (bytes <= have) return cudaSuccess;
-  const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (e == cudaSuccess) have = bytes;
-  return e;
-}
-
-int num_sms() {
-  static const int n = [] {
-    int dev = 0, v = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
-    return v > 0 ? v : 152;
-  }();
-  return n;
-}
-
 static bool is_pow2(int v) { return v > 0 && (v & (v - 1)) == 0; }
 
 // Grid, nodes and potential of §2 from the ABI problem (float64 on the host).

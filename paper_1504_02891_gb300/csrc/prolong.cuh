@@ -192,16 +192,18 @@ static gpe_status launch_prolong_line_t(int axis, ProlongArgs<T> A, int nbatch, 
   if (axis == 0) {
     constexpr int NT = axx_threads<T>(LF), NL = NT / FFT::TPL;
     const size_t smem = (size_t)FFT::F * sizeof(typename FFT::Tw) + 2 * (size_t)NL * FFT::P * sizeof(typename FFT::X);
-    static const cudaError_t allowed = raise_smem((const void*)k_prolong_x<T, KIND, LF>, smem);
-    GPE_CUDA(allowed);
+    static KernelShape shape;
+    int occ = 0;
+    GPE_CUDA(kernel_shape(shape, (const void*)k_prolong_x<T, KIND, LF>, NT, smem, &occ));
     const long long rows = G.M / G.len, lines = KIND == LK_CPLX ? rows : (rows + 1) / 2;
     A.tiles = (int)((lines + NL - 1) / NL);
     GPE_CUDA(launch_pdl(k_prolong_x<T, KIND, LF>, nbatch * A.tiles, NT, smem, st, A));
   } else {
     constexpr int CW = axs_cw<T>(LF), NT = axs_threads<T>(LF);
     const size_t smem = (size_t)FFT::F * sizeof(typename FFT::Tw) + 2 * (size_t)FFT::F * CW * sizeof(typename FFT::X);
-    static const cudaError_t allowed = raise_smem((const void*)k_prolong_s<T, KIND, LF>, smem);
-    GPE_CUDA(allowed);
+    static KernelShape shape;
+    int occ = 0;
+    GPE_CUDA(kernel_shape(shape, (const void*)k_prolong_s<T, KIND, LF>, NT, smem, &occ));
     A.width = axis == 1 ? G.n0 : G.n0 * G.n1;
     A.planes_per_inst = axis == 1 ? G.n2 : 1;
     const int cols = KIND == LK_CPLX ? CW : 2 * CW;
