@@ -20,10 +20,18 @@
 // most the line's sum(|re| + |im|) = L1, so the input level m (max < 2^m) is
 // the highest that keeps every stage and the spectrum X below 2^62.  Symbol: a
 // 62-bit fraction of a power of two 2^es >= max |symbol|, lowered by k bits.
-// Inverse: with Y = symbol X, a partial sum of n values is at most
-// sqrt(n) ||Y||_2, and
-//   ||Y||_2^2 <= sigma^2 F ||x||_2^2,  ||x||_2^2 <= max(|re|, |im|) L1,
-// sigma the root mean square of the symbol; k keeps them below 2^62.
+// Inverse: a partial sum of symbol X over n frequencies, every F/n-th one, is
+// the line's product with the sum of symbol(p) e^{-2 pi i p m / F} over them, by
+// Cauchy-Schwarz at most
+//   sqrt(n F) sigma_n ||x||_2,   ||x||_2^2 <= max(|re|, |im|) L1,
+// sigma_n the root mean square of the symbol a p^2 + c p over those frequencies
+// (p in [-1, 1)).  k keeps this below 2^62 with a common
+// sigma^2 = 0.21 a^2 + 0.34 c^2 for all of them.  sigma_n^2 is at most 1.03 (n >=
+// 64), 1.09 (32), 1.5 (8) and 2.17 (4) times that, all with a c < 0 and the
+// Nyquist frequency among the n (over all offsets, F = 32 to 1024), so values
+// stay below 2^62.3 between stages, and a sum of the two parts of a four-term
+// sum inside a radix-8 butterfly below 2^62.6; sums, halves and products hold
+// up to 2^63.
 // Rounding happens where bits are dropped, so it is about one unit of the
 // largest spectrum value (2^-61 L1) per spectrum value, where float64
 // transforms round every operation to 2^-53 of its own size.  Data and factor
@@ -57,7 +65,7 @@ __device__ __forceinline__ long long madw(int a, int b, long long c) {
 }
 __device__ __forceinline__ long long mulw(int a, int b) { return (long long)a * (long long)b; }
 
-// a w / 2^62, w = (wh, wl) in balanced halves; |a| < 2^62.5.
+// a w / 2^62, w = (wh, wl) in balanced halves; |a| < 2^62.6.
 __device__ __forceinline__ long long fix_mul(long long a, int wh, int wl) {
   int ah, al;
   split_balanced(a, ah, al);
@@ -301,9 +309,9 @@ struct LineFFT<double, LF> {
     const double a = sym.c2 * (sym.dl * pm) * (sym.dl * pm), c = sym.c1c * (sym.dl * pm);
     const bool rot = c != 0.0;
     const int es = dexp(fabs(a) + fabs(c)) - 1022;
-    // ||Y||_2^2 <= 2^R2 in the spectrum's units; mean square of the symbol
-    // (a p^2 + c p over p in [-1, 1)): a^2/5 + c^2/3, and a little more on
-    // short lines.  Later radix-8 stages grow by 1.5 bits and drop 2
+    // F sigma^2 ||x||_2^2 <= 2^R2 in the spectrum's units; sigma^2 is a^2/5 + c^2/3
+    // (the mean square over p in [-1, 1)) and a little more.  Later radix-8
+    // stages grow by 1.5 bits and drop 2
     const int R2 = LF + (L.m - LOW) + (L.m + L.l - LOW) + dexp(0.21 * a * a + 0.34 * c * c) - 1022 - 2 * es;
     const int k = max(0, max((R2 + 4) >> 1, ((R2 + LF + 1) >> 1) - LOW) - 62);
     // a, c as fractions of 2^(62 - k): mantissas shifted from 2^(E - 1075)
