@@ -164,7 +164,9 @@ typedef struct {
                          (sine: real fields) queue their line kernels instead  [1] */
   int cluster;        /* float32 Algorithm 1 on 2D Fourier grids: one thread-block
                          cluster holds the whole state in distributed shared
-                         memory (grids up to 256^2 complex)                      [1] */
+                         memory (grids up to 256^2; with `persistent`, Algorithm 1
+                         on 256^2 complex grids outside gpe_solve_batch runs in
+                         its cooperative launch)                                 [1] */
   int search;         /* line search of every Algorithm 1 run: 0 the nonmonotone
                          search of Eq. NMLS-Armijo from half a BB step (Eq. bb-1);
                          1 the monotone Armijo search of the Remark after

@@ -16,19 +16,20 @@
 //   k_axis_x: NL lines per CTA, the threads of a line consecutive.
 //
 // The odd half of a sine line is mirrored through the exchange buffer, so each
-// value is read from memory once.  The operands of the epilogue are fetched
-// (registers in float32, cp.async slots in float64) before the transforms, or
-// on large float64 grids after them (see launch_axis_x_t).
+// value is read from memory once.  The accumulator and V are fetched (registers
+// in float32, cp.async slots in float64) before the transforms, or on large
+// float64 grids after them (see launch_axis_x_t); the other vectors of the
+// epilogue after them, those of several values ahead of their stores.
 //
 // What bounds them: on 128^3 grids the arrays stay in L2 and the integer and
 // float32 issue counts (half of the cycles of the strided kernels, with 32% of
 // the warps resident in float32 and 23% in float64); on 64^3 a kernel is a
 // chain of a few latencies.
 // Measured against the general passes (a shared-memory tile per axis): 127^3
-// sine gradient float64 1039 -> 208 us, Hessian-vector float32 117 -> 46 us
+// sine gradient float64 1039 -> 208 us, Hessian-vector float32 117 -> 41.4 us
 // (245 and 59 before the register budget below, the two-level folds and the
-// programmatic launches), energy of 512 points float64 52 -> 26.5 us (with the
-// pinned sums).
+// programmatic launches; 45.6 before the epilogue's operands were gathered),
+// energy of 512 points float64 52 -> 27.6 us (with the pinned sums).
 #pragma once
 #include "lines2d.cuh"
 
@@ -47,7 +48,9 @@ template <typename T> __host__ __device__ constexpr int axs_threads(int lf) { re
 // Resident CTAs the strided kernel's registers are sized for: 24 warps per SM in
 // float32 (85 registers) and 16 in float64 (128), where the compiler's own
 // choice (92 and 168) left room for 16 and 12 (127^3: Hessian-vector float32
-// 48.5 -> 45.6 us, gradient float64 217 -> 208).
+// 48.5 -> 45.6 us, gradient float64 217 -> 208; measured there, on 256-point
+// transforms, only).  CTAs of 512 (float64: 256) threads, the longest lines, are
+// left to the compiler.
 template <typename T> __host__ __device__ constexpr int axs_minb(int lf) {
   const int warps = sizeof(T) == 4 ? 24 : 16, w = axs_threads<T>(lf) / 32;
   return axs_threads<T>(lf) >= (sizeof(T) == 4 ? 512 : 256) ? 1 : warps / w;
@@ -58,7 +61,7 @@ template <typename T> __host__ __device__ constexpr int axx_threads(int lf) {
   const int base = sizeof(T) == 4 ? 128 : 64;
   return (1 << lf) / 8 > base ? (1 << lf) / 8 : base;
 }
-// registers: 128 per thread, except the float64 strided kernel
+// registers: at most 128 per thread
 template <typename T> __host__ __device__ constexpr int axx_minb(int lf) { return 65536 / (axx_threads<T>(lf) * 128); }
 
 // Mirror a sine line: this thread's points s < 4 (m = j + s F/8 in [0, N), the
@@ -434,13 +437,14 @@ static gpe_status launch_axis_x_t(const GridDev<T>& d, const PassData<T>& D, int
   // float64: shared-memory slots for the epilogue's operands hide their latency
   // behind the transforms, but cost resident CTAs.  With more than two and a half
   // waves of groups the operands are loaded after the transforms instead (128^3
-  // real Fourier gradient 165 -> 147 us, 127^3 sine gradient 208.4 -> 206.5 and
-  // Hessian-vector 188.6 -> 186.2; at 2.2 waves, four 64^3 complex gradients,
-  // 151 against 153, at 1.6, three 64^3 sine gradients, 114 against 122)
+  // real Fourier gradient 165 -> 147.5 us, 127^3 sine gradient 209.8 -> 207.0 and
+  // Hessian-vector 187.5 -> 182.1; at 2.2 waves, four 64^3 complex gradients,
+  // 151 with and without, at 1.6, three 64^3 sine gradients, 116 against 124)
   const int slots = sizeof(T) == 8 && 2LL * groups * nbatch <= 5LL * occ_all * num_sms();
   const size_t smem = slots ? all : few;
   // one resident wave (each CTA pays its tables and a reduction of its sums; a
-  // CTA per group took 47.8 us for the 127^3 Hessian-vector product, this 45.6),
+  // CTA per group took 47.8 us for the 127^3 Hessian-vector product, this 45.6
+  // then),
   // within the reduction scratch
   long long cap = std::min<long long>((long long)(slots ? occ_all : occ_few) * num_sms(), d.max_blocks);
   const int tiles = (int)std::max<long long>(1, std::min<long long>(groups, std::max<long long>(cap / nbatch, 1)));

@@ -12,9 +12,11 @@
 // the passes themselves count, take the same time both ways (81 against 84 us).
 //
 // Every value that another CTA writes during the launch is read from L2
-// (ld.global.cg); X^k, P_k, V and the tables are constant.  CTAs of 256 threads
-// (128 on 256-point lines, which gives 256^2 grids 64 CTAs) hold 256 threads /
-// (F/8) complex lines, so 64^3 grids take one tile per CTA and axis.
+// (ld.global.cg); X^k, P_k, V and the tables are constant while it is resident
+// (a cooperative launch has plain edges).  CTAs of 256 threads (128 on 256-point
+// lines: chosen on 256^2 grids, where it gives 64 CTAs; 127^3 sine grids, whose
+// lines are as long, were only measured with it) hold their threads / (F/8)
+// complex lines, so 64^3 grids take one tile per CTA and axis.
 #pragma once
 #include "lines3.cuh"
 
