@@ -19,16 +19,16 @@
 // value is read from memory once.  The accumulator and V are fetched (registers
 // in float32, cp.async slots in float64) before the transforms, or on large
 // float64 grids after them (see launch_axis_x_t); the other vectors of the
-// epilogue after them, those of several values ahead of their stores.
+// epilogue after them, ahead of the line's stores.
 //
 // What bounds them: on 128^3 grids the arrays stay in L2 and the integer and
 // float32 issue counts (half of the cycles of the strided kernels, with 32% of
 // the warps resident in float32 and 23% in float64); on 64^3 a kernel is a
 // chain of a few latencies.
 // Measured against the general passes (a shared-memory tile per axis): 127^3
-// sine gradient float64 1039 -> 208 us, Hessian-vector float32 117 -> 41.4 us
+// sine gradient float64 1039 -> 208 us, Hessian-vector float32 117 -> 40.8 us
 // (245 and 59 before the register budget below, the two-level folds and the
-// programmatic launches; 45.6 before the epilogue's operands were gathered),
+// programmatic launches; 45.6 with the stores between the epilogue's loads),
 // energy of 512 points float64 52 -> 27.6 us (with the pinned sums).
 #pragma once
 #include "lines2d.cuh"
@@ -379,17 +379,27 @@ __global__ void __launch_bounds__(axx_threads<T>(LF), axx_minb<T>(LF)) k_axis_x(
       }
     }
     const bool diff = epilogue_diff(E);
-    constexpr int NB = epi_batch<V, EPI>(NV);   // values whose vectors are loaded ahead of their stores
+    // with other vectors to load, the results take the linear part's place and
+    // are stored last: a load must not wait for the store of the value before
+    // it, and gathering the loads of several values ahead of their stores spills
+    // (64^2 real float32 F 22.1 us gathered, 19.0 stored last; 64^3 sine 21.7 and
+    // 19.8; 128 x 64 x 32 float64 F 47 and 45.3, its first evaluation, which loads
+    // nothing, 38.9 and 40.9)
+    constexpr bool LATE = epi_nops(EPI) > 0;
 #pragma unroll
-    for (int q0 = 0; q0 < NV; q0 += NB) {
-      EpiOps<V, EPI> o[NB];
+    for (int q = 0; q < NV; ++q)
+      if (has(q)) {
+        EpiOps<V, EPI> o;
+        epilogue_load<T, CPLX, EPI, 0>(o, E, ibase + at(q));
+        if constexpr (LATE)
+          epilogue_put<T, CPLX, EPI>(E, value(q), part(q), o, acc, amax, diff, [&](V g) { part(q) = g; });
+        else
+          epilogue_apply<T, CPLX, EPI>(E, ibase + at(q), value(q), part(q), o, acc, amax, diff);
+      }
+    if constexpr (LATE && EPI != EPI_RATIO) {
 #pragma unroll
-      for (int u = 0; u < NB; ++u)
-        if (has(q0 + u)) epilogue_load<T, CPLX, EPI, 1>(o[u], E, ibase + at(q0 + u));
-#pragma unroll
-      for (int u = 0; u < NB; ++u)
-        if (has(q0 + u))
-          epilogue_apply<T, CPLX, EPI>(E, ibase + at(q0 + u), value(q0 + u), part(q0 + u), o[u], acc, amax, diff);
+      for (int q = 0; q < NV; ++q)
+        if (has(q)) E.out[ibase + at(q)] = part(q);
     }
   }
   if (EPI == EPI_HESS || D.nq == 0) return;

@@ -905,21 +905,21 @@ __device__ __forceinline__ void epilogue_load(EpiOps<typename VT<T, CPLX>::V, EP
   }
 }
 
-// One point: output and sums.  diff (objective passes): there is a current
+// One point: the output, handed to put, and the sums.  diff (objective passes): there is a current
 // point.  A run's first evaluation has none and its control reads no difference
 // sum (slots Q_SS.. and Q_MAX); in float64 they are half of the 36 operations a
 // point, of which an SM sub-partition issues one warp's in 64 clocks: they were
 // 37 of the 80 thousand cycles of the 256^2 real x-kernel (49 -> 44.5 us without
 // the differences).
-template <typename T, bool CPLX, int EPI, typename A>
-__device__ __forceinline__ void epilogue_apply(const EpiCtx<T, CPLX>& E, long long gi, typename VT<T, CPLX>::V x,
-                                               typename VT<T, CPLX>::V lin,
-                                               const EpiOps<typename VT<T, CPLX>::V, EPI>& o, A (&acc)[NQ], T& amax,
-                                               bool diff) {
+template <typename T, bool CPLX, int EPI, typename A, typename Put>
+__device__ __forceinline__ void epilogue_put(const EpiCtx<T, CPLX>& E, typename VT<T, CPLX>::V x,
+                                             typename VT<T, CPLX>::V lin,
+                                             const EpiOps<typename VT<T, CPLX>::V, EPI>& o, A (&acc)[NQ], T& amax,
+                                             bool diff, Put&& put) {
   using V = typename VT<T, CPLX>::V;
   if constexpr (EPI == EPI_GRAD) {
     const T x2 = tre(x, x);
-    if (E.out) E.out[gi] = lin + (E.nl * x2) * x;
+    if (E.out) put(lin + (E.nl * x2) * x);
     acc_add(acc[0], tre(x, lin));
     acc_add(acc[1], x2 * x2);
     acc_add(acc[2], x2);
@@ -928,7 +928,7 @@ __device__ __forceinline__ void epilogue_apply(const EpiCtx<T, CPLX>& E, long lo
     const T p2 = tre(p, p);
     const T R = tre(p, x);
     // gathered by x and p: 12 operations a complex point instead of 18 (float64 issues 2 a clock)
-    E.out[gi] = lin + (E.nl * p2 + E.shift) * x + (T(2) * E.nl * R) * p;
+    put(lin + (E.nl * p2 + E.shift) * x + (T(2) * E.nl * R) * p);
   } else if constexpr (EPI == EPI_RATIO) {
     const V d = x;
     const V xk = o.v[0], gk = o.v[1];
@@ -958,7 +958,7 @@ __device__ __forceinline__ void epilogue_apply(const EpiCtx<T, CPLX>& E, long lo
       const T d2 = tre(dd, dd);
       acc_add(acc[Q_WX], T(4) * E.nl * x2 * R + T(2) * E.nl * (x2 * d2 + T(2) * R * R) + T(0.5) * E.delta * d2);
     }
-    E.out[gi] = g;
+    put(g);
     const T y2 = tre(y, y);
     acc_add(acc[Q_E2], tre(y, lin));
     acc_add(acc[Q_E4], y2 * y2);
@@ -995,7 +995,7 @@ __device__ __forceinline__ void epilogue_apply(const EpiCtx<T, CPLX>& E, long lo
     const T x2 = tre(xk, xk), R = tre(xk, y);
     const V hD = E.lin_scale * lin + (T(4) * E.nl) * (x2 * y + (T(2) * R) * xk);
     const V gh = pk + hD + (E.delta - E.thk) * y;
-    E.out[gi] = gh;
+    put(gh);
     const V X = xk + y;
     acc_add(acc[Q_WX], tre(pk, y) + E.thk * R + T(0.5) * tre(y, hD) + T(0.5) * E.delta * tre(y, y));
     acc_add(acc[Q_NY], tre(X, X));
@@ -1015,6 +1015,14 @@ __device__ __forceinline__ void epilogue_apply(const EpiCtx<T, CPLX>& E, long lo
     acc_add(acc[Q_DF], tre(s, q) - T(0.5) * tre(s, v));   // the model is quadratic: trapezoid exact
     amax = fmax(amax, s2);
   }
+}
+// The output stored at once.
+template <typename T, bool CPLX, int EPI, typename A>
+__device__ __forceinline__ void epilogue_apply(const EpiCtx<T, CPLX>& E, long long gi, typename VT<T, CPLX>::V x,
+                                               typename VT<T, CPLX>::V lin,
+                                               const EpiOps<typename VT<T, CPLX>::V, EPI>& o, A (&acc)[NQ], T& amax,
+                                               bool diff) {
+  epilogue_put<T, CPLX, EPI>(E, x, lin, o, acc, amax, diff, [&](typename VT<T, CPLX>::V g) { E.out[gi] = g; });
 }
 
 // The first evaluation of a float64 run leaves out the difference sums.
@@ -1364,7 +1372,7 @@ __global__ void __launch_bounds__(NTHREADS) k_alg1_persist(PersistArgs<T> P) {
 // points.  The difference is taken before it is scaled: its rounding is that of
 // the neighbours' sum alone.  With one diagonal (V + sum 1/h^2) x for all axes
 // the kernel was two operations a point and 4 us shorter (149 x 100 x 76: 71.2
-// against 75.3 us), but its error 2 to 2.5 times as large on smooth states of
+// against 76 us), but its error 2 to 2.5 times as large on smooth states of
 // two and three dimensions (against extended precision; scaling each x and
 // neighbours' sum by itself lies between).
 template <typename T, bool CPLX, int EPI>
